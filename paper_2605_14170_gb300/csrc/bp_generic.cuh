@@ -16,9 +16,9 @@
 // (__fadd_rn / __fmul_rn) in the order the oracle uses: variable sums in
 // ascending row order of H^(t) excluding the own edge, sum-product phi sums
 // in ascending column order excluding the own edge.  Min-sum takes its min
-// over the other edges and MBBP_LMAX from prefix and suffix minima (exact),
-// then one correctly rounded alpha product per edge.  Signs come from the
-// sign bits: the LLRs enter as mu + 0 (turning -0 into +0) and every q is a
+// over the other edges and MBBP_LMAX, and their sign product, from prefix and
+// suffix folds (exact), then one correctly rounded alpha product per edge.
+// Signs come from the sign bits: the LLRs enter as mu + 0 (turning -0 into +0) and every q is a
 // sum that starts from mu, so no q is -0 and its sign bit is set exactly
 // when q < 0, the oracle's sign rule.  Hence normalized min-sum reproduces
 // the FP32 oracle bit for bit; sum-product differs only through
@@ -61,28 +61,14 @@ template <int DC, int RULE>
 __device__ __forceinline__ void check_out(const float (&q)[DC], float* msg, int r, int MP, int deg,
                                           uint32_t sbit, float alpha) {
     if (RULE == MBBP_RULE_NMS) {
-        // sign parity of the row (syndrome bit included) from the sign bits
-        uint32_t sx = sbit << 31;
+        // alpha carries the syndrome's sign, the excluded minimum that of the
+        // other edges
+        const float sa = __uint_as_float(__float_as_uint(alpha) ^ (sbit << 31));
+        float x[DC];
+        excluded_min<DC>(q, x);
 #pragma unroll
-        for (int j = 0; j < DC; ++j) sx ^= __float_as_uint(q[j]);
-        sx &= 0x80000000u;
-        // min over the other edges and LMAX: prefix and suffix minima
-        float pre[DC], suf[DC];
-        pre[0] = MBBP_LMAX;
-#pragma unroll
-        for (int j = 1; j < DC; ++j) pre[j] = fminf(pre[j - 1], fabsf(q[j - 1]));
-        suf[DC - 1] = MBBP_LMAX;
-#pragma unroll
-        for (int j = DC - 2; j >= 0; --j)
-            suf[j] = (j == DC - 2) ? fabsf(q[DC - 1]) : fminf(suf[j + 1], fabsf(q[j + 1]));
-#pragma unroll
-        for (int j = 0; j < DC; ++j) {
-            if (j < deg) {
-                const float excl = (j == DC - 1) ? pre[j] : (j == 0 ? fminf(MBBP_LMAX, suf[0]) : fminf(pre[j], suf[j]));
-                const uint32_t mag = __float_as_uint(__fmul_rn(alpha, excl));
-                msg[j * MP + r] = __uint_as_float(mag ^ ((sx ^ __float_as_uint(q[j])) & 0x80000000u));
-            }
-        }
+        for (int j = 0; j < DC; ++j)
+            if (j < deg) msg[j * MP + r] = __fmul_rn(sa, x[j]);
     } else {
         // sum-product with Gallager's phi: |m| = phi(sum_{k != j} phi(|q_k|))
         float f[DC];

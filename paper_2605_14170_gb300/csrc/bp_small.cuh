@@ -58,31 +58,25 @@ __device__ __forceinline__ void check_row(char* smc, const float (&q)[K], const 
                                           int k, int deg, bool valid, uint32_t sbit, float alpha,
                                           float* tr, const int32_t* se, int MP) {
     const int lane = threadIdx.x & 31;
-    uint32_t sx = sbit << 31;
-#pragma unroll
-    for (int j = 0; j < K; ++j) sx ^= __float_as_uint(q[j]);
-    sx &= 0x80000000u;
     if (RULE == MBBP_RULE_NMS) {
-        // min over the other edges and LMAX, from prefix and suffix minima
-        float pre[K], suf[K];
-        pre[0] = MBBP_LMAX;
-#pragma unroll
-        for (int j = 1; j < K; ++j) pre[j] = fminf(pre[j - 1], fabsf(q[j - 1]));
-        suf[K - 1] = MBBP_LMAX;
-#pragma unroll
-        for (int j = K - 2; j >= 0; --j)
-            suf[j] = (j == K - 2) ? fabsf(q[K - 1]) : fminf(suf[j + 1], fabsf(q[j + 1]));
+        // alpha carries the syndrome's sign, the excluded minimum that of the
+        // other edges
+        const float sa = __uint_as_float(__float_as_uint(alpha) ^ (sbit << 31));
+        float x[K];
+        excluded_min<K>(q, x);
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            const float excl = (j == K - 1) ? pre[j] : (j == 0 ? fminf(MBBP_LMAX, suf[0]) : fminf(pre[j], suf[j]));
-            const uint32_t mag = __float_as_uint(__fmul_rn(alpha, excl));
-            const uint32_t out = mag ^ ((sx ^ __float_as_uint(q[j])) & 0x80000000u);
+            const float out = __fmul_rn(sa, x[j]);
             if (valid && (REG || j < deg)) {
-                sts(smc, cb[j] + 128 * k, __uint_as_float(out));
-                if (TRACE && tr) tr[__ldg(se + j * MP + ((lane + slot_rot(j)) & 31) + 32 * k)] = __uint_as_float(out);
+                sts(smc, cb[j] + 128 * k, out);
+                if (TRACE && tr) tr[__ldg(se + j * MP + ((lane + slot_rot(j)) & 31) + 32 * k)] = out;
             }
         }
     } else {
+        uint32_t sx = sbit << 31;
+#pragma unroll
+        for (int j = 0; j < K; ++j) sx ^= __float_as_uint(q[j]);
+        sx &= 0x80000000u;
         float f[K];
 #pragma unroll
         for (int j = 0; j < K; ++j) f[j] = (REG || j < deg) ? phi(fabsf(q[j])) : 0.0f;

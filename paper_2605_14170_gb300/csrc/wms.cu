@@ -168,26 +168,16 @@ __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const u
         float qq[DC];
 #pragma unroll
         for (int j = 0; j < DC; ++j) qq[j] = (j < deg) ? q[j * MP + r] : MBBP_LMAX;
-        // the min over the other edges (and LMAX) from prefix and suffix
-        // minima, the sign parity from the sign bits (no q is -0: the LLRs
-        // enter as mu + 0), both exact
-        uint32_t sx = ((sb >> k) & 1u) << 31;
-#pragma unroll
-        for (int j = 0; j < DC; ++j) sx ^= __float_as_uint(qq[j]);
-        sx &= 0x80000000u;
-        float pre[DC], suf[DC];
-        pre[0] = MBBP_LMAX;
-#pragma unroll
-        for (int j = 1; j < DC; ++j) pre[j] = fminf(pre[j - 1], fabsf(qq[j - 1]));
-        suf[DC - 1] = MBBP_LMAX;
-#pragma unroll
-        for (int j = DC - 2; j >= 0; --j)
-            suf[j] = (j == DC - 2) ? fabsf(qq[DC - 1]) : fminf(suf[j + 1], fabsf(qq[j + 1]));
+        // the min over the other edges (and LMAX) with their sign product
+        // (no q is -0: the LLRs enter as mu + 0), exact; the syndrome's sign
+        // joins below
+        const uint32_t sx = ((sb >> k) & 1u) << 31;
+        float x[DC];
+        excluded_min<DC>(qq, x);
 #pragma unroll
         for (int j = 0; j < DC; ++j) {
             if (j >= deg) continue;
-            const float mn = (j == DC - 1) ? pre[j] : (j == 0 ? fminf(MBBP_LMAX, suf[0]) : fminf(pre[j], suf[j]));
-            const float smn = __uint_as_float(__float_as_uint(mn) ^ ((sx ^ __float_as_uint(qq[j])) & 0x80000000u));
+            const float smn = __uint_as_float(__float_as_uint(x[j]) ^ sx);
             float wj, gg;
             if constexpr (SLOT) {
                 const float2 p = __ldg(reinterpret_cast<const float2*>(wt) + j * MP + r);
