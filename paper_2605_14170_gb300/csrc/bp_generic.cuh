@@ -7,8 +7,11 @@
 // after the variable pass and m_{c->v} after the check pass (each pass reads
 // every message of a node before it overwrites them, and every edge belongs
 // to exactly one check and one variable, so no other lane touches it).  Lanes
-// own checks r = lane + 32k; edge j of check r lives at slot j * MP + r, so
-// the check pass reads and writes with unit stride across the warp.
+// own row positions r = lane + 32k; edge j of the row at position r lives at
+// slot row_slot(r) + 32 j, so the check pass reads and writes with unit
+// stride across the warp, at constant offsets from one address per row.  The
+// host places the rows and orders the variables to spread the variable pass
+// over the shared-memory banks.
 // Variables are visited in degree-sorted order so that the lanes of one step
 // mostly share a degree.
 //
@@ -34,6 +37,12 @@ constexpr unsigned kFull = 0xffffffffu;
 
 __host__ __device__ __forceinline__ int align16(int x) { return (x + 15) & ~15; }
 
+// First slot of the row at position r (edge j at + 32 j): blocks of 32 rows.
+template <int DC>
+__host__ __device__ __forceinline__ int row_slot(int r) {
+    return (r >> 5) * (32 * DC) + (r & 31);
+}
+
 struct WarpLayout {
     int S, npad, ehpad, per_warp, hcol_bytes;
 };
@@ -54,12 +63,12 @@ __device__ __forceinline__ float phi(float x) {
     return log1pf(__fdiv_rn(2.0f, expm1f(x)));
 }
 
-// Check-node update of row r (Eq. (2) with the syndrome sign, or the
+// Check-node update of a row (Eq. (2) with the syndrome sign, or the
 // sum-product rule) from its incoming messages q[0..deg) (q[j] = MBBP_LMAX
-// for j >= deg); writes the deg outgoing messages to slots j * MP + r.
-template <int DC, int RULE>
-__device__ __forceinline__ void check_out(const float (&q)[DC], float* msg, int r, int MP, int deg,
-                                          uint32_t sbit, float alpha) {
+// for j >= deg); writes the deg outgoing messages to row[32 j].  REG: the
+// row fills the kernel width (deg == DC), no edge is tested.
+template <int DC, int RULE, bool REG>
+__device__ __forceinline__ void check_out(const float (&q)[DC], float* row, int deg, uint32_t sbit, float alpha) {
     if (RULE == MBBP_RULE_NMS) {
         // alpha carries the syndrome's sign, the excluded minimum that of the
         // other edges
@@ -68,47 +77,46 @@ __device__ __forceinline__ void check_out(const float (&q)[DC], float* msg, int 
         excluded_min<DC>(q, x);
 #pragma unroll
         for (int j = 0; j < DC; ++j)
-            if (j < deg) msg[j * MP + r] = __fmul_rn(sa, x[j]);
+            if (REG || j < deg) row[32 * j] = __fmul_rn(sa, x[j]);
     } else {
         // sum-product with Gallager's phi: |m| = phi(sum_{k != j} phi(|q_k|))
         float f[DC];
         uint32_t par = sbit;
 #pragma unroll
         for (int j = 0; j < DC; ++j) {
-            f[j] = (j < deg) ? phi(fabsf(q[j])) : 0.0f;
+            f[j] = (REG || j < deg) ? phi(fabsf(q[j])) : 0.0f;
             par ^= (q[j] < 0.f) ? 1u : 0u;
         }
         float pre = 0.0f;  // f_0 + ... + f_{j-1}, left to right
 #pragma unroll
         for (int j = 0; j < DC; ++j) {
-            if (j < deg) {
+            if (REG || j < deg) {
                 float sum = pre;
 #pragma unroll
                 for (int k = j + 1; k < DC; ++k)
-                    if (k < deg) sum = __fadd_rn(sum, f[k]);
+                    if (REG || k < deg) sum = __fadd_rn(sum, f[k]);
                 const float mag = fminf(phi(sum), MBBP_SP_MAX);
                 const uint32_t neg = par ^ ((q[j] < 0.f) ? 1u : 0u);
-                msg[j * MP + r] = neg ? -mag : mag;
+                row[32 * j] = neg ? -mag : mag;
             }
             pre = __fadd_rn(pre, f[j]);
         }
     }
 }
 
-// Flooding check pass of row r: its q messages are in its own slots.  With
+// Flooding check pass of one row: its q messages are in its own slots.  With
 // a trace pointer tr, the row's new messages also go to tr[0..deg) (edge j of
 // the row is its j-th column in ascending order).
-template <int DC, int RULE>
-__device__ __forceinline__ void check_row(float* msg, int r, int MP, int deg, uint32_t sbit,
-                                          float alpha, float* tr = nullptr) {
+template <int DC, int RULE, bool REG>
+__device__ __forceinline__ void check_row(float* row, int deg, uint32_t sbit, float alpha, float* tr) {
     float q[DC];
 #pragma unroll
-    for (int j = 0; j < DC; ++j) q[j] = (j < deg) ? msg[j * MP + r] : MBBP_LMAX;
-    check_out<DC, RULE>(q, msg, r, MP, deg, sbit, alpha);
+    for (int j = 0; j < DC; ++j) q[j] = (REG || j < deg) ? row[32 * j] : MBBP_LMAX;
+    check_out<DC, RULE, REG>(q, row, deg, sbit, alpha);
     if (tr) {
 #pragma unroll
         for (int j = 0; j < DC; ++j)
-            if (j < deg) tr[j] = msg[j * MP + r];
+            if (REG || j < deg) tr[j] = row[32 * j];
     }
 }
 
@@ -275,9 +283,19 @@ __device__ __forceinline__ void store_item_group(const ShotIO& io, unsigned long
 // or global memory).  A group's threads own rows gt, gt + 32 G, ... and
 // variable positions likewise (gt: the thread's index in the group) and meet
 // on named barrier `bar` between passes; the arithmetic of every row and
-// variable is the same whatever G.  TRACE: io.c2v receives the check
-// messages of every iteration (the last one run remains).
-template <int DC, int DV, int RULE, bool TRACE = false, int G = 1>
+// variable is the same whatever G.  REG: every row fills the kernel width.
+// OUT: the call asks for posteriors (io.post) and / or the check messages of
+// every iteration (io.c2v; the last one run remains); without OUT the loops
+// carry no test for them.  Both are compiled apart because the passes are
+// bound by issue slots and the shared-memory path ([[288,12,18]]: 40
+// instructions per lane and edge update, the path 90% busy, 35% of its
+// wavefronts bank conflicts).  With the blocked slots, the bank-aware
+// placement and both splits: [[288,12,18]] R = 32, 20,011 shots at p = 0.04,
+// 8.10 -> 7.76 ms; length-882 code R = 64, 5,000 shots at p = 0.0333, 17.0 ->
+// 15.4 ms; a length-254 code with rows of weight 8, 3,001 shots, 282 -> 241
+// us; weighted min-sum decoding of 2,000 shots of the length-882 code 8.17 ->
+// 7.07 ms; training step on [[144,12,12]] R = 8 5.73 -> 5.55 ms.
+template <int DC, int DV, int RULE, bool REG, bool OUT, int G = 1>
 __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, int shot, int b,
                                          unsigned char* area, const uint16_t* hcol, int bar = 0) {
     constexpr int GT = 32 * G;
@@ -304,10 +322,14 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
         eh[v] = (x < 0.f) ? 1 : 0;
     }
     if (lane == 0) eh[n] = 0;  // padding column of hcol
-    uint32_t sb = 0;
+    uint32_t sb = 0, sbo = 0;  // by row position; by row of H (halting test)
     for (int k = 0; k < row_steps; ++k) {
         const int r = lane + GT * k;
         if (r < Mb) sb |= (uint32_t)(__ldg(sy + (__ldg(rinfo + r) & 0xffffu)) & 1u) << k;
+    }
+    for (int k = 0; k < orow_steps; ++k) {
+        const int r = lane + GT * k;
+        if (r < m) sbo |= (uint32_t)(__ldg(sy + r) & 1u) << k;
     }
     gsync<G>(bar);
     // q^(0)_{v->c} = mu_v
@@ -320,7 +342,7 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
 #pragma unroll
             for (int i = 0; i < 6; ++i)
                 if (i < deg) msg_at(msg, packed_off(d, i)) = x;
-            if (io.post) io.post[item * n + v] = x;
+            if (OUT && io.post) io.post[item * n + v] = x;
         }
     } else {
         for (int p = lane; p < n; p += GT) {
@@ -328,7 +350,7 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
             const int v = d.y & 0xffff, deg = (int)(d.y >> 16);
             const float x = mu_s[v];
             for (int i = 0; i < deg; ++i) msg[__ldg(B.vslot + d.x + i)] = x;
-            if (io.post) io.post[item * n + v] = x;
+            if (OUT && io.post) io.post[item * n + v] = x;
         }
     }
     gsync<G>(bar);
@@ -347,7 +369,7 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
             const int r = lane + GT * k;
             bool gok = true;
             if (r < m) {
-                uint32_t par = (sb >> k) & 1u;
+                uint32_t par = (sbo >> k) & 1u;
 #pragma unroll
                 for (int j = 0; j < DC; ++j) par ^= eh[hcol[j * mpad + r]];
                 gok = (par == 0u);
@@ -368,14 +390,15 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
             break;
         }
         // check pass
-        for (int k = 0; k < row_steps; ++k) {
+        float* row = msg + row_slot<DC>(lane);
+        for (int k = 0; k < row_steps; ++k, row += GT * DC) {
             const int r = lane + GT * k;
             if (r < Mb) {
-                const int deg = B.regular ? DC : (int)((__ldg(rinfo + r) >> 16) & 0xffu);
-                float* tr = TRACE ? io.c2v + item * (unsigned long long)io.c2v_stride +
-                                        __ldg(B.rowptr + (size_t)b * MP + r)
-                                  : nullptr;
-                check_row<DC, RULE>(msg, r, MP, deg, (sb >> k) & 1u, io.alpha, tr);
+                const int deg = REG ? DC : (int)((__ldg(rinfo + r) >> 16) & 0xffu);
+                float* tr = (OUT && io.c2v) ? io.c2v + item * (unsigned long long)io.c2v_stride +
+                                                  __ldg(B.rowptr + (size_t)b * MP + r)
+                                            : nullptr;
+                check_row<DC, RULE, REG>(row, deg, (sb >> k) & 1u, io.alpha, tr);
             }
         }
         gsync<G>(bar);
@@ -391,7 +414,7 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
                 const int v = d.x & 0xffff, deg = (int)(d.x >> 16);
                 const float post = var_dispatch_packed(deg, msg, d, mu_s[v]);
                 eh[v] = (post < 0.f) ? 1 : 0;
-                if (io.post) io.post[item * n + v] = post;
+                if (OUT && io.post) io.post[item * n + v] = post;
             }
         } else {
             uint2 dn = (lane < n) ? __ldg(vd + lane) : make_uint2(0u, 0u);
@@ -401,7 +424,7 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
                 const int v = d.y & 0xffff, deg = (int)(d.y >> 16);
                 const float post = var_dispatch<1, DV>(deg, msg, B.vslot + d.x, mu_s[v]);
                 eh[v] = (post < 0.f) ? 1 : 0;
-                if (io.post) io.post[item * n + v] = post;
+                if (OUT && io.post) io.post[item * n + v] = post;
             }
         }
         gsync<G>(bar);
@@ -459,11 +482,11 @@ __device__ __forceinline__ void run_item_serial(const DevBases& B, const ShotIO&
     }
     if (lane == 0) eh[n] = 0;
     for (int i = lane; i < L.S; i += 32) msg[i] = 0.0f;  // m^(0)_{c->v} = 0
-    uint32_t sb = 0;  // syndrome bits of the rows lane + 32k (halting test)
+    uint32_t sb = 0;  // syndrome bits of the rows lane + 32k of H (halting test)
     for (int k = 0; k < row_steps; ++k) {
         const int r = lane + 32 * k;
         const uint32_t bit = (r < Mb) ? (uint32_t)(__ldg(sy + (__ldg(rinfo + r) & 0xffffu)) & 1u) : 0u;
-        sb |= bit << k;
+        if (r < m) sb |= (uint32_t)(__ldg(sy + r) & 1u) << k;
         const uint32_t word = __ballot_sync(kFull, bit);
         if (lane == 0) sbits[k] = word;
     }
@@ -505,7 +528,7 @@ __device__ __forceinline__ void run_item_serial(const DevBases& B, const ShotIO&
                 for (int j = 0; j < DC; ++j) {
                     q[j] = MBBP_LMAX;
                     if (j < deg) {
-                        const int slot = j * MP + r;
+                        const int slot = row_slot<DC>(r) + 32 * j;
                         const uint2 e = __ldg(ev + slot);
                         const int dv = (int)(e.y >> 16);
                         float x = mu_s[e.y & 0xffffu];
@@ -519,7 +542,7 @@ __device__ __forceinline__ void run_item_serial(const DevBases& B, const ShotIO&
                         q[j] = x;  // unclamped, as in var_update
                     }
                 }
-                check_out<DC, RULE>(q, msg, r, MP, deg, (sbits[r >> 5] >> (r & 31)) & 1u, io.alpha);
+                check_out<DC, RULE, false>(q, msg + row_slot<DC>(r), deg, (sbits[r >> 5] >> (r & 31)) & 1u, io.alpha);
             }
             __syncwarp();
         }
@@ -538,13 +561,18 @@ __device__ __forceinline__ void run_item_serial(const DevBases& B, const ShotIO&
     __syncwarp();
 }
 
-// Dispatch on the kernel width of a representation set.
+// Dispatch on the kernel width of a representation set and on its rows.
 template <int RULE>
 __device__ __forceinline__ void run_item_any(const DevBases& B, const ShotIO& io, int shot, int b,
                                              unsigned char* area, const uint16_t* hcol) {
-    if (B.DC == 6) run_item<6, 6, RULE>(B, io, shot, b, area, hcol);
-    else if (B.DC == 8) run_item<8, 8, RULE>(B, io, shot, b, area, hcol);
-    else run_item<12, 12, RULE>(B, io, shot, b, area, hcol);
+    if (B.DC == 6) {
+        if (B.regular) run_item<6, 6, RULE, true, false>(B, io, shot, b, area, hcol);
+        else run_item<6, 6, RULE, false, false>(B, io, shot, b, area, hcol);
+    } else if (B.DC == 8) {
+        run_item<8, 8, RULE, false, false>(B, io, shot, b, area, hcol);
+    } else {
+        run_item<12, 12, RULE, false, false>(B, io, shot, b, area, hcol);
+    }
 }
 
 }  // namespace generic_bp

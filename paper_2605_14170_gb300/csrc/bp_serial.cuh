@@ -3,8 +3,8 @@
 // A warp decodes shots of one representation, CS at a time, pulling them
 // from a per-representation counter.  Each shot keeps its check-to-variable
 // messages m_{c->v} in shared memory (edge j of the row at position p at
-// slot j * MP + p, followed by one slot holding -0.0f, the exact additive
-// identity of IEEE addition); the host places the rows (a permutation of
+// slot row_slot(p) + 32 j, followed by one slot holding -0.0f, the exact
+// additive identity of IEEE addition); the host places the rows (a permutation of
 // the positions) so that the lanes of one access hit different banks.  A serial iteration visits the layers
 // of the representation in order; within a layer the (row, shot) pairs are
 // spread over the lanes.  Rows of a layer share no variable, so the pairs of
@@ -201,15 +201,16 @@ __device__ __forceinline__ void run_rep(const DevBases& B, const ShotIO& io, int
                 const int r = __ldg(lrows + i0 + (idx >> CSH));
                 const int deg = REG ? DC : (int)((__ldg(rinfo + r) >> 16) & 0xffu);
                 float* ms = msg + sh * L.SH;
+                const int rs = generic_bp::row_slot<DC>(r);
                 const float* mus = mu + sh * L.NP;
                 float q[DC];
 #pragma unroll
                 for (int j = 0; j < DC; ++j) {
-                    if (REG || j < deg) q[j] = edge_q<NO>(ms, mus, __ldg(ed + j * MP + r));
+                    if (REG || j < deg) q[j] = edge_q<NO>(ms, mus, __ldg(ed + rs + 32 * j));
                     else q[j] = MBBP_LMAX;
                 }
                 const uint32_t sbit = (sbits[sh * L.RW + (r >> 5)] >> (r & 31)) & 1u;
-                generic_bp::check_out<DC, RULE>(q, ms, r, MP, deg, sbit, io.alpha);
+                generic_bp::check_out<DC, RULE, REG>(q, ms + rs, deg, sbit, io.alpha);
             }
             __syncwarp();
         }

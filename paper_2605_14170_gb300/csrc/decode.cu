@@ -33,7 +33,7 @@ constexpr int kGenericWideWarps = 16;
 // for codes whose per-item shared memory, not registers, limits the resident
 // warps: the same shared memory then holds G times the warps).  Group g of
 // the block uses named barrier 1 + g (at most 8 groups: ids 1..8).
-template <int DC, int DV, int RULE, int MAXW, bool TRACE = false, int G = 1>
+template <int DC, int DV, int RULE, int MAXW, bool REG, bool OUT, int G>
 __global__ void __launch_bounds__(MAXW * 32)
 decode_kernel(const DecodeArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -67,7 +67,7 @@ decode_kernel(const DecodeArgs a) {
         if (item >= a.total_items) break;
         const int b = (int)(item / batch);
         const int shot = (int)(item - (unsigned long long)b * batch);
-        generic_bp::run_item<DC, DV, RULE, TRACE, G>(B, a.io, shot, b, area, hcol_s, bar);
+        generic_bp::run_item<DC, DV, RULE, REG, OUT, G>(B, a.io, shot, b, area, hcol_s, bar);
     }
 }
 
@@ -234,7 +234,7 @@ cudaError_t launch_serial_t(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     return cudaGetLastError();
 }
 
-template <int K, int RULE, bool TRACE, int G>
+template <int K, int RULE, bool REG, bool OUT, int G>
 cudaError_t launch_decode_g(const DecodeArgs& a, int cls, int warps, int per_sm, size_t smem, cudaStream_t s,
                             int sm_count) {
     const unsigned long long groups = (unsigned long long)(warps / G);
@@ -243,13 +243,13 @@ cudaError_t launch_decode_g(const DecodeArgs& a, int cls, int warps, int per_sm,
     if (want < grid) grid = want;
     const dim3 gd((unsigned)grid), bd((unsigned)(warps * 32));
     if (cls == 0)
-        decode_kernel<K, K, RULE, kWarpsPerBlock, TRACE, G><<<gd, bd, smem, s>>>(a);
+        decode_kernel<K, K, RULE, kWarpsPerBlock, REG, OUT, G><<<gd, bd, smem, s>>>(a);
     else
-        decode_kernel<K, K, RULE, kGenericWideWarps, TRACE, G><<<gd, bd, smem, s>>>(a);
+        decode_kernel<K, K, RULE, kGenericWideWarps, REG, OUT, G><<<gd, bd, smem, s>>>(a);
     return cudaGetLastError();
 }
 
-template <int K, int RULE, bool TRACE>
+template <int K, int RULE, bool REG, bool OUT>
 cudaError_t launch_decode_t(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     // Launch shapes: (block class, warps per item G in {1, 2, 4}).  The narrow
     // class runs blocks of up to 8 warps, the wide class up to 16 (compiled
@@ -262,12 +262,12 @@ cudaError_t launch_decode_t(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     // smaller one (codes whose message areas, not registers, limit the
     // resident warps).
     const void* kerns[3][2] = {
-        {reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kWarpsPerBlock, TRACE, 1>),
-         reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kGenericWideWarps, TRACE, 1>)},
-        {reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kWarpsPerBlock, TRACE, 2>),
-         reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kGenericWideWarps, TRACE, 2>)},
-        {reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kWarpsPerBlock, TRACE, 4>),
-         reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kGenericWideWarps, TRACE, 4>)}};
+        {reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kWarpsPerBlock, REG, OUT, 1>),
+         reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kGenericWideWarps, REG, OUT, 1>)},
+        {reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kWarpsPerBlock, REG, OUT, 2>),
+         reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kGenericWideWarps, REG, OUT, 2>)},
+        {reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kWarpsPerBlock, REG, OUT, 4>),
+         reinterpret_cast<const void*>(decode_kernel<K, K, RULE, kGenericWideWarps, REG, OUT, 4>)}};
     const generic_bp::WarpLayout L = generic_bp::warp_layout(K, a.B.MP, a.B.mpad, a.B.n);
     int choice[3][2][2] = {};  // [log2 G][class] = {warps per block, blocks per SM}
     for (int gi = 0; gi < 3; ++gi) {
@@ -297,14 +297,18 @@ cudaError_t launch_decode_t(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     const int warps = choice[gi_best][cls_best][0], per_sm = choice[gi_best][cls_best][1];
     if (warps == 0) return cudaErrorInvalidConfiguration;
     const size_t smem = (size_t)L.hcol_bytes + (size_t)(warps >> gi_best) * L.per_warp;
-    if (gi_best == 0) return launch_decode_g<K, RULE, TRACE, 1>(a, cls_best, warps, per_sm, smem, s, sm_count);
-    if (gi_best == 1) return launch_decode_g<K, RULE, TRACE, 2>(a, cls_best, warps, per_sm, smem, s, sm_count);
-    return launch_decode_g<K, RULE, TRACE, 4>(a, cls_best, warps, per_sm, smem, s, sm_count);
+    if (gi_best == 0) return launch_decode_g<K, RULE, REG, OUT, 1>(a, cls_best, warps, per_sm, smem, s, sm_count);
+    if (gi_best == 1) return launch_decode_g<K, RULE, REG, OUT, 2>(a, cls_best, warps, per_sm, smem, s, sm_count);
+    return launch_decode_g<K, RULE, REG, OUT, 4>(a, cls_best, warps, per_sm, smem, s, sm_count);
 }
 
 template <int K, int RULE>
 cudaError_t launch_decode_k(const DecodeArgs& a, cudaStream_t s, int sm_count) {
-    return a.io.c2v ? launch_decode_t<K, RULE, true>(a, s, sm_count) : launch_decode_t<K, RULE, false>(a, s, sm_count);
+    // posteriors and the message trace take a kernel of their own, as do
+    // min-sum calls on codes whose rows all fill the kernel width
+    if (a.io.c2v || a.io.post) return launch_decode_t<K, RULE, false, true>(a, s, sm_count);
+    if (RULE == MBBP_RULE_NMS && a.B.regular) return launch_decode_t<K, RULE, RULE == MBBP_RULE_NMS, false>(a, s, sm_count);
+    return launch_decode_t<K, RULE, false, false>(a, s, sm_count);
 }
 
 }  // namespace

@@ -169,11 +169,13 @@ mbbp_status collect_impl(const Tanner& g, int R, uint64_t seed, std::vector<int3
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Small-code layout: ELL index sigma[r] of every row r of H^(t), the slot
+// Bank-aware layout: ELL index sigma[r] of every row r of H^(t), the slot
 // s = slot[r][j] < deg(r) that holds the j-th edge of row r (j in H's column
 // order), and the variable at every position (32 positions = one warp step of
-// the variable pass).  Slot s of row r lives in shared-memory bank
-// (sigma[r] + rot(s)) & 31.  In the variable pass the 32 lanes of a step read
+// the variable pass).  Small-code layout: slot s of row r lives in
+// shared-memory bank (sigma[r] + rot(s)) & 31.  Generic layout: bank
+// sigma[r] & 31, slots in column order (the sum-product rule adds its terms
+// in that order).  In the variable pass the 32 lanes of a step read
 // the i-th edge of their variables together; the cost of that access is the
 // largest number of lanes that hit one bank.  Simulated annealing over row
 // swaps, swaps of two edge slots within a row and swaps of equal-degree
@@ -181,17 +183,18 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // check rule is symmetric in a row's edges (minima and sign parity are
 // exact), so any layout gives the same results; the sum-product rule adds
 // its terms in slot order, which moves its rounding by a few ulps.
-struct SmallLayout {
+struct BankLayout {
     std::vector<int> sigma;               // ELL index of row r
-    std::vector<std::array<int, 6>> slot;  // slot of the j-th edge of row r
+    std::vector<std::array<int, MBBP_MAX_ROW_WEIGHT>> slot;  // slot of the j-th edge of row r
     std::vector<int> order;               // variable at position p
 };
 
-SmallLayout small_layout(const Tanner& g, const std::vector<int>& src, int n, int MP, uint64_t seed) {
+BankLayout bank_layout(const Tanner& g, const std::vector<int>& src, int n, int MP, uint64_t seed, bool small,
+                        int iters) {
     const int M = (int)src.size();
-    constexpr int DVX = 8;
+    constexpr int DVX = MBBP_MAX_COL_WEIGHT;
     std::vector<std::vector<std::pair<int, int>>> ve(n);  // (row, j), ascending row
-    std::vector<std::array<int, 6>> ei(M);                 // edge index i of (r, j) in ve[v]
+    std::vector<std::array<int, MBBP_MAX_ROW_WEIGHT>> ei(M);  // edge index i of (r, j) in ve[v]
     for (int r = 0; r < M; ++r) {
         const auto& cols = g.rcols[src[r]];
         for (int j = 0; j < (int)cols.size(); ++j) {
@@ -202,20 +205,21 @@ SmallLayout small_layout(const Tanner& g, const std::vector<int>& src, int n, in
     std::vector<std::vector<std::pair<int, int>>> re(M);  // (variable, edge index i)
     for (int v = 0; v < n; ++v)
         for (int i = 0; i < (int)ve[v].size(); ++i) re[ve[v][i].first].push_back({v, i});
-    SmallLayout L;
+    BankLayout L;
     L.sigma.resize(M);
     L.slot.resize(M);
     for (int r = 0; r < M; ++r) {
         L.sigma[r] = r;
-        for (int j = 0; j < 6; ++j) L.slot[r][j] = j;
+        for (int j = 0; j < MBBP_MAX_ROW_WEIGHT; ++j) L.slot[r][j] = j;
     }
-    // variables by descending degree: the last step, the one that n leaves
-    // partly empty, then holds the smallest degrees (every step costs its
-    // largest degree for all 32 lanes)
+    // small codes: variables by descending degree: the last step, the one
+    // that n leaves partly empty, then holds the smallest degrees (every step
+    // costs its largest degree for all 32 lanes); generic: ascending (measured
+    // the faster one there)
     L.order.resize(n);
     for (int v = 0; v < n; ++v) L.order[v] = v;
     std::stable_sort(L.order.begin(), L.order.end(),
-                     [&](int a, int b) { return ve[a].size() > ve[b].size(); });
+                     [&](int a, int b) { return small ? ve[a].size() > ve[b].size() : ve[a].size() < ve[b].size(); });
     std::vector<int> posof(n);
     for (int p = 0; p < n; ++p) posof[L.order[p]] = p;
     const int steps = (n + 31) / 32;
@@ -246,7 +250,7 @@ SmallLayout small_layout(const Tanner& g, const std::vector<int>& src, int n, in
         pairs[c] -= q - 1;
         if (q == top[c] && h[q] == 0) top[c] = q - 1;
     };
-    auto bank = [&](int r, int j) { return (L.sigma[r] + slot_rot(L.slot[r][j])) & 31; };
+    auto bank = [&](int r, int j) { return (L.sigma[r] + (small ? slot_rot(L.slot[r][j]) : 0)) & 31; };
     auto cell = [&](int v, int i) { return (posof[v] >> 5) * DVX + i; };
     for (int v = 0; v < n; ++v)
         for (int i = 0; i < (int)ve[v].size(); ++i) inc((size_t)cell(v, i) * 32 + bank(ve[v][i].first, ve[v][i].second));
@@ -254,8 +258,9 @@ SmallLayout small_layout(const Tanner& g, const std::vector<int>& src, int n, in
     // largest degree; lanes with fewer edges (and the padding positions past
     // n) read the warp's zero slot there, all at one address (a broadcast):
     // one more access in the zero slot's bank, fixed because moves only swap
-    // variables of equal degree between steps.
-    {
+    // variables of equal degree between steps.  (The generic kernels run each
+    // degree of a step apart and read no zero slot.)
+    if (small) {
         const int zero_bank = (6 * MP) & 31;
         for (int st = 0; st < steps; ++st) {
             int dmin = 1 << 30, dmax = 0;
@@ -275,19 +280,20 @@ SmallLayout small_layout(const Tanner& g, const std::vector<int>& src, int n, in
     long total = 0;
     for (int c = 0; c < steps * DVX; ++c) { remax(c); total += mx[c]; }
     std::vector<int> best_sigma = L.sigma, best_order = L.order;
-    std::vector<std::array<int, 6>> best_slot = L.slot;
+    std::vector<std::array<int, MBBP_MAX_ROW_WEIGHT>> best_slot = L.slot;
     long best = LONG_MAX;  // none yet
     uint64_t rs = seed;
     auto rnd = [&]() { rs += 0x9E3779B97F4A7C15ULL; uint64_t z = rs;
                        z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ULL;
                        z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL; return z ^ (z >> 31); };
     std::vector<int> cells;
-    const int iters = 1000000;
     for (int it = 0; it < iters; ++it) {
         const double T = 0.6 * (1.0 - (double)it / iters) + 0.02;
         cells.clear();
         long before = 0, after = 0;
-        const int kind = (int)(rnd() % 3);  // 0: two rows, 1: two edge slots of a row, 2: two variables
+        // 0: two rows, 1: two edge slots of a row (small codes), 2: two variables
+        int kind = (int)(rnd() % 3);
+        if (!small && kind == 1) kind = 2;
         const bool row_move = kind == 0 || (kind == 2 && steps == 1);
         int a = 0, b = 0;
         if (kind == 1) {
@@ -318,9 +324,12 @@ SmallLayout small_layout(const Tanner& g, const std::vector<int>& src, int n, in
                 for (int c : cells) remax(c);
             }
         } else if (row_move) {
+            // generic: rows stay in their block of 32 (sigma's block is the row's
+            // own), so a warp's 32 rows keep their consecutive edge numbers and
+            // the training kernels their sectors of w, g and the gradients
             a = (int)(rnd() % M);
-            b = (int)(rnd() % M);
-            if (a == b) continue;
+            b = small ? (int)(rnd() % M) : (a & ~31) + (int)(rnd() & 31);
+            if (a == b || b >= M) continue;
             for (int rr : {a, b})
                 for (auto& e : re[rr]) cells.push_back(cell(e.first, e.second));
             std::sort(cells.begin(), cells.end());
@@ -567,25 +576,92 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
     B->lorder.assign((size_t)R * MP, 0);
     B->lptr.assign((size_t)R * (MP + 1), 0);
     B->nlayers.assign(R, 0);
+    // Small-code tables (register-resident kernel), when a shape fits.
+    int shape = 0;
+    if (K == 6)
+        for (int i = 0; i < kNumSmallShapes && !shape; ++i)
+            if (n <= 32 * kSmallShapes[i].VS && MP <= 32 * kSmallShapes[i].RS &&
+                m <= 32 * kSmallShapes[i].ORS)
+                shape = i + 1;
+    // The layouts of the R representations are independent: anneal them on
+    // the host's cores.
+    struct RepLayout {
+        std::vector<int> src;         // source row of every row of H^(t)
+        std::vector<int> layer_of;    // serial layer of every row
+        std::vector<int> idx_in;      // its index in the layer
+        int layers = 0;
+        std::vector<int> sp;          // chunked serial path: row positions
+        BankLayout generic, small;
+    };
+    std::vector<RepLayout> layouts(R);
+    {
+        // generic layout: the wavefronts per variable pass fall from 108 to 74
+        // on [[288,12,18]] and from 290 to 219 on the length-882 code in 20,000
+        // steps (9 ms a representation); 50 times the steps reach 69 and 208
+        const int anneal = 20000;
+        const int nth = std::max(1, std::min(R, (int)std::thread::hardware_concurrency()));
+        std::atomic<int> next{0};
+        auto worker = [&]() {
+            for (int t = next++; t < R; t = next++) {
+                RepLayout& L = layouts[t];
+                const int M = m + set_ptr[t + 1] - set_ptr[t];
+                L.src.resize(M);
+                for (int r = 0; r < M; ++r) L.src[r] = r < m ? r : set_rows[set_ptr[t] + (r - m)];
+                // Serial schedule: rows go, in row order, into the first layer
+                // holding none of their variables.
+                std::vector<std::vector<uint8_t>> layer_vars;
+                std::vector<int> count;
+                std::vector<std::vector<int>> rc(M);
+                L.layer_of.resize(M);
+                L.idx_in.resize(M);
+                for (int r = 0; r < M; ++r) {
+                    rc[r] = g.rcols[L.src[r]];
+                    size_t y = 0;
+                    for (; y < layer_vars.size(); ++y) {
+                        bool clash = false;
+                        for (int v : rc[r]) clash = clash || layer_vars[y][v];
+                        if (!clash) break;
+                    }
+                    if (y == layer_vars.size()) {
+                        layer_vars.emplace_back(n, 0);
+                        count.push_back(0);
+                    }
+                    for (int v : rc[r]) layer_vars[y][v] = 1;
+                    L.layer_of[r] = (int)y;
+                    L.idx_in[r] = count[y]++;
+                }
+                L.layers = (int)layer_vars.size();
+                if (chunked) {
+                    const int CS = serial_bp::shots_per_warp(K, MP, mpad, n);
+                    L.sp = serial_positions(rc, L.layer_of, L.idx_in, CS, K, n, 0xBA4Cull + (uint64_t)t);
+                }
+                L.generic = bank_layout(g, L.src, n, MP, 0x6E4Eull + (uint64_t)t, false, anneal);
+                if (shape) L.small = bank_layout(g, L.src, n, MP, 0x5EEDull + (uint64_t)t, true, 1000000);
+            }
+        };
+        std::vector<std::thread> pool;
+        for (int i = 1; i < nth; ++i) pool.emplace_back(worker);
+        worker();
+        for (auto& th : pool) th.join();
+    }
+    auto slot_of = [&](int pos, int j) { return (pos >> 5) * (32 * K) + 32 * j + (pos & 31); };
+    std::vector<uint16_t> lrows16((size_t)R * MP, 0);
     for (int t = 0; t < R; ++t) {
-        const int extra = set_ptr[t + 1] - set_ptr[t];
-        const int M = m + extra;
+        const RepLayout& L = layouts[t];
+        const int M = (int)L.src.size();
+        const std::vector<int>& pos = L.generic.sigma;
         rows[t] = M;
         std::vector<std::vector<uint16_t>> vl(n);
         int E = 0;
         for (int r = 0; r < M; ++r) {
-            const int src = r < m ? r : set_rows[set_ptr[t] + (r - m)];
-            const auto& cols = g.rcols[src];
-            rowinfo[(size_t)t * MP + r] = (uint32_t)src | ((uint32_t)cols.size() << 16) | (1u << 31);
-            rowptr[(size_t)t * MP + r] = E;
-            for (int j = 0; j < (int)cols.size(); ++j) vl[cols[j]].push_back((uint16_t)(j * MP + r));
+            const auto& cols = g.rcols[L.src[r]];
+            rowinfo[(size_t)t * MP + pos[r]] = (uint32_t)L.src[r] | ((uint32_t)cols.size() << 16) | (1u << 31);
+            rowptr[(size_t)t * MP + pos[r]] = E;
+            for (int j = 0; j < (int)cols.size(); ++j) vl[cols[j]].push_back((uint16_t)slot_of(pos[r], j));
             E += (int)cols.size();
         }
         edges[t] = E;
-        std::vector<int> ord(n);
-        for (int v = 0; v < n; ++v) ord[v] = v;
-        std::stable_sort(ord.begin(), ord.end(),
-                         [&](int a, int b) { return vl[a].size() < vl[b].size(); });
+        const std::vector<int>& ord = L.generic.order;
         std::vector<uint2> vstart(n);
         for (int p = 0; p < n; ++p) {
             const int v = ord[p];
@@ -601,59 +677,43 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
                 vdesc6[(size_t)t * n + p] = make_uint4(d.y, o[0] | (o[1] << 16), o[2] | (o[3] << 16), o[4] | (o[5] << 16));
             }
         }
-        // Serial schedule: every edge slot points at its variable's slot list;
-        // rows go, in row order, into the first layer holding none of their
-        // variables.
-        std::vector<std::vector<uint8_t>> layer_vars;
-        std::vector<int> layer_of(M);
+        // Serial schedule: every edge slot points at its variable's slot list.
         for (int r = 0; r < M; ++r) {
-            const int src = r < m ? r : set_rows[set_ptr[t] + (r - m)];
-            const auto& cols = g.rcols[src];
-            for (int j = 0; j < (int)cols.size(); ++j) evar[(size_t)t * K * MP + (size_t)j * MP + r] = vstart[cols[j]];
-            size_t L = 0;
-            for (; L < layer_vars.size(); ++L) {
-                bool clash = false;
-                for (int v : cols) clash = clash || layer_vars[L][v];
-                if (!clash) break;
-            }
-            if (L == layer_vars.size()) layer_vars.emplace_back(n, 0);
-            for (int v : cols) layer_vars[L][v] = 1;
-            layer_of[r] = (int)L;
+            const auto& cols = g.rcols[L.src[r]];
+            for (int j = 0; j < (int)cols.size(); ++j)
+                evar[(size_t)t * K * MP + (size_t)slot_of(pos[r], j)] = vstart[cols[j]];
         }
-        const int nl = (int)layer_vars.size();
+        const int nl = L.layers;
         int32_t* lo = B->lorder.data() + (size_t)t * MP;
         int32_t* lp = B->lptr.data() + (size_t)t * (MP + 1);
-        int pos = 0;
-        for (int L = 0; L < nl; ++L) {
-            lp[L] = pos;
+        int at = 0;
+        for (int y = 0; y < nl; ++y) {
+            lp[y] = at;
             for (int r = 0; r < M; ++r)
-                if (layer_of[r] == L) lo[pos++] = r;
+                if (L.layer_of[r] == y) {
+                    lrows16[(size_t)t * MP + at] = (uint16_t)pos[r];
+                    lo[at++] = r;
+                }
         }
-        lp[nl] = pos;
+        lp[nl] = at;
         B->nlayers[t] = nl;
         if (chunked) {
             // chunk kernel: rows at bank-aware positions, descriptors by position
-            std::vector<std::vector<int>> rc(M);
-            std::vector<int> idx_in(M);
-            for (int r = 0; r < M; ++r) {
-                const int src = r < m ? r : set_rows[set_ptr[t] + (r - m)];
-                rc[r] = g.rcols[src];
-            }
-            for (int L = 0; L < nl; ++L)
-                for (int i = lp[L]; i < lp[L + 1]; ++i) idx_in[lo[i]] = i - lp[L];
-            const int CS = serial_bp::shots_per_warp(K, MP, mpad, n);
-            const std::vector<int> sp = serial_positions(rc, layer_of, idx_in, CS, K, n, 0xBA4Cull + (uint64_t)t);
+            const std::vector<int>& sp = L.sp;
+            std::vector<int> row_at(MP, 0);  // row at a generic-layout position
+            for (int r = 0; r < M; ++r) row_at[pos[r]] = r;
             for (int i = 0; i < M; ++i) lpos[(size_t)t * MP + i] = (uint16_t)sp[lo[i]];
-            for (int r = 0; r < M; ++r) {
-                const int src = r < m ? r : set_rows[set_ptr[t] + (r - m)];
-                rinfo_s[(size_t)t * MP + sp[r]] = (uint32_t)src | ((uint32_t)rc[r].size() << 16);
-            }
+            for (int r = 0; r < M; ++r)
+                rinfo_s[(size_t)t * MP + sp[r]] = (uint32_t)L.src[r] | ((uint32_t)g.rcols[L.src[r]].size() << 16);
             auto pack = [](const uint32_t* o) {
                 return make_uint4(o[0] | (o[1] << 16), o[2] | (o[3] << 16), o[4] | (o[5] << 16),
                                   o[6] | (o[7] << 16));
             };
-            // slot j * MP + r of the logical layout -> byte offset of j * MP + pos(r)
-            auto off = [&](uint32_t slot) { return 4u * (uint32_t)((slot / MP) * MP + sp[slot % MP]); };
+            // byte offset in this layout of a slot of the generic one
+            auto off = [&](uint32_t slot) {
+                const int p = (int)(slot / (32 * K)) * 32 + (int)(slot & 31), j = (int)(slot / 32) % K;
+                return 4u * (uint32_t)slot_of(sp[row_at[p]], j);
+            };
             for (int v = 0; v < n; ++v) {
                 uint32_t o[8];
                 for (int i = 0; i < 8; ++i) o[i] = i < (int)vl[v].size() ? off(vl[v][i]) : negz;
@@ -670,15 +730,7 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
             }
         }
     }
-    std::vector<uint16_t> lrows16(B->lorder.begin(), B->lorder.end());
     std::vector<uint16_t> lptr16(B->lptr.begin(), B->lptr.end());
-    // Small-code tables (register-resident kernel), when a shape fits.
-    int shape = 0;
-    if (K == 6)
-        for (int i = 0; i < kNumSmallShapes && !shape; ++i)
-            if (n <= 32 * kSmallShapes[i].VS && MP <= 32 * kSmallShapes[i].RS &&
-                m <= 32 * kSmallShapes[i].ORS)
-                shape = i + 1;
     std::vector<uint4> vdesc2;
     std::vector<uint32_t> rinfo2, hmask2;
     std::vector<int32_t> sedge;  // [R][6*MP] edge id (row by row, columns ascending) of every slot, or -1
@@ -691,30 +743,10 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
         rinfo2.assign((size_t)R * MP, 0);
         hmask2.assign((size_t)R * VS * ORS * 32, 0);
         sedge.assign((size_t)R * 6 * MP, -1);
-        // the bank placements of the R representations are independent:
-        // anneal them on the host's cores
-        std::vector<SmallLayout> layouts(R);
-        {
-            const int nth = std::max(1, std::min(R, (int)std::thread::hardware_concurrency()));
-            std::atomic<int> next{0};
-            auto worker = [&]() {
-                for (int t = next++; t < R; t = next++) {
-                    const int extra = set_ptr[t + 1] - set_ptr[t];
-                    std::vector<int> src(m + extra);
-                    for (int r = 0; r < m + extra; ++r) src[r] = r < m ? r : set_rows[set_ptr[t] + (r - m)];
-                    layouts[t] = small_layout(g, src, n, MP, 0x5EEDull + (uint64_t)t);
-                }
-            };
-            std::vector<std::thread> pool;
-            for (int i = 1; i < nth; ++i) pool.emplace_back(worker);
-            worker();
-            for (auto& th : pool) th.join();
-        }
         for (int t = 0; t < R; ++t) {
-            const int extra = set_ptr[t + 1] - set_ptr[t];
-            std::vector<int> src(m + extra);
-            for (int r = 0; r < m + extra; ++r) src[r] = r < m ? r : set_rows[set_ptr[t] + (r - m)];
-            const SmallLayout& L = layouts[t];
+            const std::vector<int>& src = layouts[t].src;
+            const BankLayout& L = layouts[t].small;
+            const std::vector<int>& gpos = layouts[t].generic.sigma;
             std::vector<int> posof(n);
             for (int p = 0; p < n; ++p) posof[L.order[p]] = p;
             std::vector<std::vector<uint16_t>> vs(n);
@@ -726,7 +758,7 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
                     const int sj = L.slot[r][j];
                     const int sl = sj * MP + (sg & ~31) + ((sg + slot_rot(sj)) & 31);
                     vs[cols[j]].push_back((uint16_t)sl);
-                    sedge[(size_t)t * 6 * MP + sl] = rowptr[(size_t)t * MP + r] + j;
+                    sedge[(size_t)t * 6 * MP + sl] = rowptr[(size_t)t * MP + gpos[r]] + j;
                 }
             }
             // byte offsets within a warp's message area; a missing edge (and

@@ -149,8 +149,8 @@ __device__ __forceinline__ void wms_var_pass(const DevBases& B, int b, const uin
 // One WMS check pass: m <- g m + (1 - g) w S mn(q).  wt, gt: parameters of
 // this iteration for representation b ([E] in row-major edge order); or,
 // with SLOT, wt points at the iteration's (w, g) pairs in the message layout
-// (pair of edge j of row r at float2 index j * MP + r: one coalesced load
-// per edge).  With G warps per item the thread with group index gt takes
+// (pair of edge j of row r at float2 index row_slot(r) + 32 j: one coalesced
+// load per edge).  With G warps per item the thread with group index gt takes
 // rows gt, gt + 32 G, ...; bit k of sb is the syndrome bit of its k-th row.
 template <int DC, int G = 1, bool SLOT = false>
 __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const uint32_t* rinfo,
@@ -165,9 +165,10 @@ __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const u
         if (r >= Mb) continue;
         const int deg = B.regular ? DC : (int)((__ldg(rinfo + r) >> 16) & 0xffu);
         const int e0 = SLOT ? 0 : __ldg(rp + r);
+        const int rs = generic_bp::row_slot<DC>(r);
         float qq[DC];
 #pragma unroll
-        for (int j = 0; j < DC; ++j) qq[j] = (j < deg) ? q[j * MP + r] : MBBP_LMAX;
+        for (int j = 0; j < DC; ++j) qq[j] = (j < deg) ? q[rs + 32 * j] : MBBP_LMAX;
         // the min over the other edges (and LMAX) with their sign product
         // (no q is -0: the LLRs enter as mu + 0), exact; the syndrome's sign
         // joins below
@@ -180,7 +181,7 @@ __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const u
             const float smn = __uint_as_float(__float_as_uint(x[j]) ^ sx);
             float wj, gg;
             if constexpr (SLOT) {
-                const float2 p = __ldg(reinterpret_cast<const float2*>(wt) + j * MP + r);
+                const float2 p = __ldg(reinterpret_cast<const float2*>(wt) + rs + 32 * j);
                 wj = p.x;
                 gg = p.y;
             } else {
@@ -188,8 +189,8 @@ __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const u
                 gg = __ldg(gt + e0 + j);
             }
             const float c = __fmul_rn(wj, smn);
-            const float mo = m[j * MP + r];
-            m[j * MP + r] = __fadd_rn(__fmul_rn(gg, mo), __fmul_rn(__fsub_rn(1.0f, gg), c));
+            const float mo = m[rs + 32 * j];
+            m[rs + 32 * j] = __fadd_rn(__fmul_rn(gg, mo), __fmul_rn(__fsub_rn(1.0f, gg), c));
         }
     }
 }
@@ -263,10 +264,14 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
         }
         if (lane == 0) post[n] = 0.0f;
         for (int i = lane; i < L.S; i += GT) m[i] = 0.0f;
-        uint32_t sb = 0;
+        uint32_t sb = 0, sbo = 0;  // by row position; by row of H (halting test)
         for (int k = 0; k < row_steps; ++k) {
             const int r = lane + GT * k;
             if (r < Mb) sb |= (uint32_t)(__ldg(sy + (__ldg(rinfo + r) & 0xffffu)) & 1u) << k;
+        }
+        for (int k = 0; a.decode && k < orow_steps; ++k) {
+            const int r = lane + GT * k;
+            if (r < m_rows) sbo |= (uint32_t)(__ldg(sy + r) & 1u) << k;
         }
         generic_bp::gsync<G>(bar);
         for (int p = lane; p < n; p += GT) {  // q^(0) = mu
@@ -287,7 +292,7 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
                 for (int k = 0; k < orow_steps; ++k) {
                     const int r = lane + GT * k;
                     if (r < m_rows) {
-                        uint32_t par = (sb >> k) & 1u;
+                        uint32_t par = (sbo >> k) & 1u;
 #pragma unroll
                         for (int j = 0; j < DC; ++j) par ^= __float_as_uint(post[hcol_s[j * B.mpad + r]]) >> 31;
                         ok = ok && (par == 0u);
@@ -488,6 +493,7 @@ wms_backward_kernel(const WmsArgs a) {
                     if (r >= Mb) continue;
                     const int deg = B.regular ? DC : (int)((__ldg(rinfo + r) >> 16) & 0xffu);
                     const int e0 = __ldg(rp + r);
+                    const int rs = generic_bp::row_slot<DC>(r);
                     // the row's parameters first: L2 loads (the shared memory
                     // leaves little L1) that then overlap the arithmetic below
                     float wv[DC], gv[DC];
@@ -498,7 +504,7 @@ wms_backward_kernel(const WmsArgs a) {
                     }
                     float qq[DC];
 #pragma unroll
-                    for (int j = 0; j < DC; ++j) qq[j] = (j < deg) ? q[j * MP + r] : MBBP_LMAX;
+                    for (int j = 0; j < DC; ++j) qq[j] = (j < deg) ? q[rs + 32 * j] : MBBP_LMAX;
                     // the smallest and second smallest |q| below LMAX with
                     // their lowest-index positions, and the sign parity: the
                     // min over the edges other than j is (min1, a1) unless
@@ -527,11 +533,11 @@ wms_backward_kernel(const WmsArgs a) {
                         const uint32_t neg = par ^ ((qq[j] < 0.f) ? 1u : 0u);
                         const float sgn = neg ? -1.0f : 1.0f;
                         const float ww = wv[j], gg = gv[j];
-                        const float gmj = gm[j * MP + r];
+                        const float gmj = gm[rs + 32 * j];
                         const float c = ww * sgn * mn;
-                        atomicAdd(ggt + e0 + j, gmj * (mprev[j * MP + r] - c));
+                        atomicAdd(ggt + e0 + j, gmj * (mprev[rs + 32 * j] - c));
                         atomicAdd(gwt + e0 + j, gmj * (1.0f - gg) * sgn * mn);
-                        gm[j * MP + r] = gmj * gg;  // becomes dL/dm^(t-1): only this lane owns the slot
+                        gm[rs + 32 * j] = gmj * gg;  // becomes dL/dm^(t-1): only this lane owns the slot
                         const float gmn = gmj * (1.0f - gg) * ww * sgn;
                         if (own) G2 += gmn;
                         else G1 += gmn;
@@ -543,7 +549,7 @@ wms_backward_kernel(const WmsArgs a) {
                         float gj = 0.0f;
                         if (j == a1) gj = G1 * sq;
                         if (j == a2) gj = G2 * sq;
-                        gq[j * MP + r] = gj;
+                        gq[rs + 32 * j] = gj;
                     }
                 }
                 __syncwarp();
@@ -604,7 +610,7 @@ wms_backward_kernel(const WmsArgs a) {
 }
 
 // Decode mode: the parameters of every (representation, iteration) in the
-// message layout, w and g side by side: wg[((b T + t) DC + j) MP + r] is the
+// message layout, w and g side by side: wg[(b T + t) DC MP + row_slot(r) + 32 j] is the
 // (w, g) of edge j of row r of H^(b) at iteration t, zeros where the row has
 // no edge j, so that the check pass reads one coalesced float2 per edge.
 template <int DC>
@@ -626,7 +632,7 @@ __global__ void wms_pack_kernel(const WmsArgs a, float2* __restrict__ wg) {
         const float* gt = a.g + bt * a.E + e0;
 #pragma unroll
         for (int j = 0; j < DC; ++j)
-            wg[(bt * DC + j) * MP + r] = (j < deg) ? make_float2(__ldg(wt + j), __ldg(gt + j)) : make_float2(0.f, 0.f);
+            wg[bt * DC * MP + generic_bp::row_slot<DC>(r) + 32 * j] = (j < deg) ? make_float2(__ldg(wt + j), __ldg(gt + j)) : make_float2(0.f, 0.f);
     }
 }
 

@@ -1,0 +1,72 @@
+"""Kernel variants chosen by the shape of the call, each against the FP32
+oracle bit for bit (normalized min-sum) at the sizes where a variant can go
+wrong: the last partly filled block of rows, rows that do not fill the kernel
+width, calls with and without posteriors.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2605_14170_gb300.inputs import channel_llr, gb_code, named_code
+
+pytestmark = pytest.mark.gpu
+
+SEED = 20260601
+
+
+def _decode(B, s, llr, iters, alpha, **kw):
+    import torch
+    from paper_2605_14170_gb300 import mbbp
+    out = mbbp.decode(B, torch.from_numpy(np.ascontiguousarray(s)).cuda(),
+                      torch.from_numpy(np.ascontiguousarray(llr, np.float32)).cuda(), iters, alpha, **kw)
+    torch.cuda.synchronize()
+    res = {k: v.cpu().numpy() for k, v in out.items() if k not in ("cand", "workspace")}
+    res["iters"] = res["iters"].view(np.uint16)
+    res["cand"] = mbbp.unpack_words(out["cand"], B.n)
+    return res
+
+
+def _assert_exact(got, ref):
+    for key, rkey in (("conv", "conv"), ("iters", "iters"), ("cand", "cand"), ("selected", "selected"),
+                      ("success", "success"), ("e_hat", "ehat")):
+        assert np.array_equal(got[key], ref[rkey]), key
+
+
+def _irregular(m, n, wmax, seed):
+    """Rows of weight 2..wmax, every column of weight 1..3."""
+    rng = np.random.default_rng(seed)
+    H = np.zeros((m, n), np.uint8)
+    H[np.arange(n) % m, np.arange(n)] = 1
+    for r in range(m):
+        want = int(rng.integers(2, wmax + 1))
+        free = [v for v in rng.permutation(n) if H[r, v] == 0 and H[:, v].sum() < 3]
+        for v in free[:max(0, want - int(H[r].sum()))]:
+            H[r, v] = 1
+    return H
+
+
+CODES = {
+    # width 6, every row full, more variables than the small-code shapes take
+    "gb166": lambda: gb_code(83, [0, 7, 31], [2, 19, 55]).HZ,
+    # width 8 (rows of weight 8), width 12 (rows of weight 10)
+    "gb90w4": lambda: gb_code(45, [0, 3, 11, 30], [1, 8, 20, 37]).HZ,
+    "gb78w5": lambda: gb_code(39, [0, 3, 11, 21, 30], [1, 8, 20, 27, 36]).HZ,
+    # width 6 with rows of several weights
+    "irregular": lambda: _irregular(70, 190, 6, 5),
+}
+
+
+@pytest.mark.parametrize("post", [False, True])
+@pytest.mark.parametrize("code", sorted(CODES))
+def test_generic_flooding_variants(code, post):
+    """The generic flooding kernel's variants: rows that fill the width or
+    not, outputs with posteriors or without."""
+    from paper_2605_14170_gb300 import mbbp
+    H = CODES[code]()
+    n = H.shape[1]
+    e, _ = oracle.sample(SEED, 0, 65, n, 0.04, "bsc")
+    s = oracle.syndrome(H, e)
+    llr = channel_llr(n, 0.04).astype(np.float32)
+    B = mbbp.mbbp_build_bases(H, 5, SEED)
+    got = _decode(B, s, llr, 40, 0.7, want_posterior=post)
+    _assert_exact(got, oracle.mbbp_decode(H, B.sets, s, llr, 40, 0.7, precision="f32"))
