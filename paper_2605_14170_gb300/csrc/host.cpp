@@ -1504,27 +1504,40 @@ size_t mbbp_wms_decode_workspace_size(const mbbp_bases* B, int batch, int T) {
     return mbbp_decode_workspace_size(B, batch) + align256((size_t)B->R * T * B->dev.DC * B->MP * 8);
 }
 
-size_t mbbp_wms_workspace_size(const mbbp_bases* B, int batch, int T, int ckpt) {
-    if (!B || batch < 0 || T < 1 || ckpt < 1) return 0;
+namespace {
+
+// Workspace of the training kernels: a work counter, the checkpoints, the
+// recomputed states of one segment per block or warp of the backward grid.
+struct WmsWorkspace {
+    size_t ckpt, seg, total;  // byte offsets; total
+};
+
+WmsWorkspace wms_workspace(const mbbp_bases* B, int batch, int T, int ckpt, bool lanes) {
     const size_t nckpt = (size_t)((T - 1) / ckpt);
+    WmsWorkspace w;
+    w.ckpt = 256;
+    if (lanes) {
+        w.seg = w.ckpt + align256(wms_lanes_ckpt_floats(B->dev, batch) * nckpt * 4);
+        w.total = w.seg + align256(wms_lanes_grid(B->dev, batch, B->sm_count) * ckpt * wms_lanes_state_floats(B->dev) * 4);
+        return w;
+    }
     const size_t S = (size_t)B->dev.DC * B->MP;
+    w.seg = w.ckpt + align256((size_t)batch * B->R * nckpt * S * 4);
     // per-warp segment buffers only when the backward pass cannot keep the
     // segment states in shared memory
-    const size_t seg = wms_states_in_smem(B->dev, ckpt) ? 0 : align256((size_t)kWmsMaxWarps * ckpt * S * 4);
-    return 256 + align256((size_t)batch * B->R * nckpt * S * 4) + seg;
+    w.total = w.seg + (wms_states_in_smem(B->dev, ckpt) ? 0 : align256((size_t)kWmsMaxWarps * ckpt * S * 4));
+    return w;
 }
 
-namespace {
-// The per-warp segment buffers (null when the backward pass keeps the
-// segment states in shared memory and the workspace has no such region).
-float* wms_seg_buf(const mbbp_bases* B, int batch, int T, int ckpt, void* workspace) {
-    if (wms_states_in_smem(B->dev, ckpt)) return nullptr;
-    const size_t nckpt = (size_t)((T - 1) / ckpt);
-    const size_t S = (size_t)B->dev.DC * B->MP;
-    return reinterpret_cast<float*>(static_cast<char*>(workspace) + 256 +
-                                    align256((size_t)batch * B->R * nckpt * S * 4));
-}
 }  // namespace
+
+size_t mbbp_wms_workspace_size(const mbbp_bases* B, int batch, int T, int ckpt) {
+    if (!B || batch < 0 || T < 1 || ckpt < 1) return 0;
+    // the one-shot-per-lane kernels take shared LLRs only, so that the LLR
+    // stride, which this size does not know, decides between the two
+    const size_t base = wms_workspace(B, batch, T, ckpt, false).total;
+    return wms_lanes_fit(B->dev, batch) ? std::max(base, wms_workspace(B, batch, T, ckpt, true).total) : base;
+}
 
 mbbp_status mbbp_wms_forward(const mbbp_bases* B, int batch, const uint8_t* syndromes, const float* llr,
                              int llr_stride, int T, const float* w, const float* g, int ckpt,
@@ -1557,9 +1570,11 @@ mbbp_status mbbp_wms_forward(const mbbp_bases* B, int batch, const uint8_t* synd
     a.counter = static_cast<unsigned long long*>(workspace);
     a.ckpt_buf = a.nckpt ? reinterpret_cast<float*>(static_cast<char*>(workspace) + 256) : nullptr;
     a.total_items = (unsigned long long)batch * B->R;
+    const bool lanes = llr_stride == 0 && wms_lanes_fit(B->dev, batch);
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e = cudaMemsetAsync(a.counter, 0, 8, s);
-    if (e == cudaSuccess) e = launch_wms(a, false, s, B->sm_count);
+    if (e == cudaSuccess)
+        e = lanes ? launch_wms_lanes(a, batch, false, s, B->sm_count) : launch_wms(a, false, s, B->sm_count);
     return e == cudaSuccess ? MBBP_OK : cuda_fail(e, "mbbp_wms_forward");
 }
 
@@ -1591,13 +1606,16 @@ mbbp_status mbbp_wms_backward(const mbbp_bases* B, int batch, const uint8_t* syn
     a.post = const_cast<float*>(posterior);
     a.gw = gw;
     a.gg = gg;
-    a.seg_buf = wms_seg_buf(B, batch, T, ckpt, workspace);
+    const bool lanes = llr_stride == 0 && wms_lanes_fit(B->dev, batch);
+    const WmsWorkspace ws = wms_workspace(B, batch, T, ckpt, lanes);
+    a.seg_buf = ws.total > ws.seg ? reinterpret_cast<float*>(static_cast<char*>(workspace) + ws.seg) : nullptr;
     a.counter = static_cast<unsigned long long*>(workspace);
     a.ckpt_buf = a.nckpt ? reinterpret_cast<float*>(static_cast<char*>(workspace) + 256) : nullptr;
     a.total_items = (unsigned long long)batch * B->R;
     cudaStream_t s = (cudaStream_t)stream;
     cudaError_t e = cudaMemsetAsync(a.counter, 0, 8, s);
-    if (e == cudaSuccess) e = launch_wms(a, true, s, B->sm_count);
+    if (e == cudaSuccess)
+        e = lanes ? launch_wms_lanes(a, batch, true, s, B->sm_count) : launch_wms(a, true, s, B->sm_count);
     return e == cudaSuccess ? MBBP_OK : cuda_fail(e, "mbbp_wms_backward");
 }
 

@@ -255,6 +255,14 @@ constexpr int kWmsMaxWarps = 152 * 16;  // warps of the backward grid (segment b
 // (then it needs no per-warp segment buffers in the workspace).
 bool wms_states_in_smem(const DevBases& B, int ckpt);
 cudaError_t launch_wms(const WmsArgs& a, bool backward, cudaStream_t s, int sm_count);
+// The one-shot-per-lane training kernels (wms_lanes.cu; shared LLRs only):
+// whether a code and batch fit them, blocks of the largest grid, floats of one
+// checkpoint of every block of shots and of one state of one block.
+bool wms_lanes_fit(const DevBases& B, int batch);
+size_t wms_lanes_grid(const DevBases& B, int batch, int sm_count);
+size_t wms_lanes_ckpt_floats(const DevBases& B, int batch);
+size_t wms_lanes_state_floats(const DevBases& B);
+cudaError_t launch_wms_lanes(const WmsArgs& a, int batch, bool backward, cudaStream_t s, int sm_count);
 // Fills a.wg-style packed parameters from a.w / a.g (a.T iterations).
 cudaError_t launch_wms_pack(const WmsArgs& a, float2* wg, cudaStream_t s, int sm_count);
 cudaError_t launch_adam(float* p, const float* g, float* m1, float* m2, size_t count, float lr, float b1,

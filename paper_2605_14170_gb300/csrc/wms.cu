@@ -9,8 +9,10 @@
 // Loss of an item: scale * sum_v BCE(sigmoid(-post_v), e_v), post = mu + sum m^(T),
 // or (all_iters) the mean of that over the posteriors of iterations 1..T.
 //
-// Kernels (generic slot layout; the backward pass one warp per (shot,
-// representation), the forward pass G warps per item, G in {1, 2, 4}):
+// Training calls with shared LLRs on codes that fit take the kernels of
+// wms_lanes.cu (one shot per lane).  Kernels here (generic slot layout; the
+// backward pass one warp per (shot, representation), the forward pass G warps
+// per item, G in {1, 2, 4}):
 //   wms_forward   T iterations, posterior, loss, a checkpoint of m every
 //                 `ckpt` iterations; or, in decode mode, the halting rule
 //                 after every iteration and the candidate for FWS
@@ -24,6 +26,7 @@
 //                 added to gw / gg with atomics;
 //   adam_step     Adam update of the parameters, clamped to [lo, hi].
 #include "bp_generic.cuh"
+#include "wms_common.cuh"
 
 namespace mbbp {
 namespace {
@@ -193,11 +196,6 @@ __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const u
             m[rs + 32 * j] = __fadd_rn(__fmul_rn(gg, mo), __fmul_rn(__fsub_rn(1.0f, gg), c));
         }
     }
-}
-
-__device__ __forceinline__ float bce_neg_sigmoid(float post, int e) {
-    const float x = e ? post : -post;
-    return x > 0.f ? x + log1pf(expf(-x)) : log1pf(expf(x));
 }
 
 // G warps decode each item together (G = 1: one warp per item; G > 1 for

@@ -70,3 +70,44 @@ def test_generic_flooding_variants(code, post):
     B = mbbp.mbbp_build_bases(H, 5, SEED)
     got = _decode(B, s, llr, 40, 0.7, want_posterior=post)
     _assert_exact(got, oracle.mbbp_decode(H, B.sets, s, llr, 40, 0.7, precision="f32"))
+
+
+@pytest.mark.parametrize("ckpt,all_iters", [(1, True), (3, False), (7, True)])
+@pytest.mark.parametrize("code", ["bb72", "gb90w4", "gb78w5", "irregular"])
+def test_wms_training_one_shot_per_lane(code, ckpt, all_iters):
+    """129 shots at R = 3: the training kernels with one shot per lane (shared
+    LLRs; a last block of one shot) against the warp-per-shot kernels, which
+    the same LLRs given per shot take.  Same posteriors bit for bit; losses
+    and gradients to the rounding of their sums: two orders of N terms differ
+    by at most 2 N 2^-24 sum|terms| (the losses' terms are of one sign and
+    added in partial sums of at most 42: 1e-5; the gradients', by norm:
+    1e-4)."""
+    import torch
+    from paper_2605_14170_gb300 import mbbp
+    H = named_code("bb72").HZ if code == "bb72" else CODES[code]()
+    n, T, batch, R = H.shape[1], 7, 129, 3
+    e, _ = oracle.sample(SEED + 1, 0, batch, n, 0.05, "bsc")
+    s = torch.from_numpy(oracle.syndrome(H, e)).cuda()
+    B = mbbp.mbbp_build_bases(H, R, SEED)
+    rng = np.random.default_rng(3)
+    E = int(B.edges.max())
+    w, g = (torch.from_numpy(rng.uniform(lo, hi, (R, T, E)).astype(np.float32)).cuda()
+            for lo, hi in ((0.4, 1.0), (0.0, 0.4)))
+    mu = torch.from_numpy(rng.uniform(1.0, 3.5, n).astype(np.float32)).cuda()
+    et = torch.from_numpy(mbbp.pack_bits(e)).cuda()
+    res = []
+    for llr in (mu, mu.repeat(batch, 1).contiguous()):
+        post = torch.full((batch, R, n), 7.0, device="cuda")
+        loss = torch.full((batch, R), 7.0, device="cuda")
+        gw, gg = torch.zeros_like(w), torch.zeros_like(g)
+        ws = torch.empty(mbbp.mbbp_wms_workspace_size(B, batch, T, ckpt), dtype=torch.uint8, device="cuda")
+        mbbp.mbbp_wms_forward(B, s, llr, T, w, g, ckpt, et, 1e-3, post, loss, ws, all_iters=all_iters)
+        mbbp.mbbp_wms_backward(B, s, llr, T, w, g, ckpt, et, 1e-3, post, gw, gg, ws, all_iters=all_iters)
+        torch.cuda.synchronize()
+        res.append([x.double().cpu().numpy() for x in (post, loss, gw, gg)])
+    (p1, l1, w1, g1), (p2, l2, w2, g2) = res
+    assert np.array_equal(p1, p2)
+    assert np.allclose(l1, l2, rtol=1e-5, atol=0)
+    for a, b in ((w1, w2), (g1, g2)):
+        assert np.linalg.norm(b) > 0
+        assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b)
