@@ -2,36 +2,57 @@
 // [[72,12,6]] and [[144,12,12]] bivariate bicycle codes of Section IV); the
 // per-chunk device code is in bp_small.cuh.  Warps pull
 // (chunk of kChunk shots, representation) work items from a global counter.
+#include <algorithm>
+
 #include "bp_small.cuh"
 
 namespace mbbp {
 namespace {
 
 constexpr int kSmallWarps = 1;  // warps per block: each warp works alone
-constexpr int kChunk = 8;       // shots per work item of a warp (same representation)
+// Work items: a run of consecutive shots of one representation.  The first
+// `s8` shots come in runs of 8, the next `s2` in runs of 2, the rest one by
+// one.  A run loads its representation's tables once, so long runs cost least
+// per shot (runs of one shot: 13% more time on [[144,12,12]] R = 16, 200,000
+// depolarizing shots at p = 0.04), but a shot that does not converge takes 100
+// iterations where most take a few, and with runs of 8 the last ones leave
+// most of the GPU idle.  So the last kTail1 shots per resident warp go one by
+// one and the kTail2 before them in pairs.  With runs of 8 throughout ->
+// this: [[72,12,6]] R = 4, 2,000 shots 106 -> 52 us; [[144,12,12]] R = 16 at
+// p = 0.0533, 300 / 2,000 / 10,000 shots 296 -> 113 / 443 -> 288 / 1308 -> 1183
+// us, 50,000 shots 5.55 -> 5.37 ms; the 200,000 shots above 11.35 -> 11.39 ms.
+// Sum-product shots cost ten times as much, their tables nothing beside: runs
+// of 2 and 1 only (4,000 shots 3.40 -> 2.76 ms).
+struct SmallWork {
+    int s8, s2, s1;
+};
+constexpr long long kTail1 = 8, kTail2 = 8;
 
 template <int VS, int RS, int ORS, int RULE, bool REG, bool OUT>
 __global__ void __launch_bounds__(kSmallWarps * 32, small_min_blocks(RS, RULE))
-decode_small_kernel(const DecodeArgs a) {
+decode_small_kernel(const DecodeArgs a, const SmallWork work) {
     extern __shared__ __align__(16) float smsg[];
     const DevBases& B = a.B;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    const int R = B.R;
+    const unsigned R = (unsigned)B.R;
     char* smc = reinterpret_cast<char*>(smsg);
     const uint32_t wbase = (uint32_t)(warp * small_bp::warp_floats(B.MP, VS, ORS) * 4);
-    const unsigned long long chunks_per_rep = ((unsigned long long)a.io.batch + kChunk - 1) / kChunk;
-    const unsigned long long total_chunks = chunks_per_rep * (unsigned long long)R;
+    const unsigned long long n8 = (unsigned long long)(work.s8 / 8) * R;
+    const unsigned long long n2 = n8 + (unsigned long long)(work.s2 / 2) * R;
+    const unsigned long long n1 = n2 + (unsigned long long)work.s1 * R;
     for (;;) {
-        unsigned long long chunk = 0;
-        if (lane == 0) chunk = atomicAdd(a.counter, 1ull);
-        chunk = __shfl_sync(small_bp::kFull, chunk, 0);
-        if (chunk >= total_chunks) break;
-        const int sblock = (int)(chunk / (unsigned long long)R);
-        const int b = (int)(chunk - (unsigned long long)sblock * R);
-        const int s0 = sblock * kChunk;
-        const int s1 = min(a.io.batch, s0 + kChunk);
-        small_bp::run_chunk<VS, RS, ORS, RULE, REG, OUT>(B, a.io, b, s0, s1, smc, wbase);
+        unsigned long long w = 0;
+        if (lane == 0) w = atomicAdd(a.counter, 1ull);
+        w = __shfl_sync(small_bp::kFull, w, 0);
+        if (w >= n1) break;
+        const int len = w < n8 ? 8 : (w < n2 ? 2 : 1);
+        const int first = w < n8 ? 0 : (w < n2 ? work.s8 : work.s8 + work.s2);
+        const unsigned long long l = w - (w < n8 ? 0 : (w < n2 ? n8 : n2));
+        const int run = (int)(l / R);
+        const int b = (int)(l - (unsigned long long)run * R);
+        const int s0 = first + run * len;
+        small_bp::run_chunk<VS, RS, ORS, RULE, REG, OUT>(B, a.io, b, s0, s0 + len, smc, wbase);
     }
 }
 
@@ -46,12 +67,18 @@ cudaError_t launch_small_t(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     int per_sm = 0;
     cudaError_t e = prepare_kernel(reinterpret_cast<const void*>(kern), warps * 32, smem, &per_sm);
     if (e != cudaSuccess) return e;
-    const unsigned long long chunks =
-        ((unsigned long long)a.io.batch + kChunk - 1) / kChunk * (unsigned long long)a.B.R;
-    unsigned long long want = (chunks + warps - 1) / warps;
     unsigned long long grid = (unsigned long long)per_sm * (unsigned long long)sm_count;
+    const long long resident = (long long)grid * warps, batch = a.io.batch, R = a.B.R;
+    SmallWork work;
+    work.s1 = (int)std::min(batch, (kTail1 * resident + R - 1) / R);
+    const long long rest = batch - work.s1;
+    work.s8 = RULE == MBBP_RULE_NMS ? (int)(std::max(0ll, rest - (kTail2 * resident + R - 1) / R) / 8 * 8) : 0;
+    work.s2 = (int)((rest - work.s8) / 2 * 2);
+    work.s1 = (int)(batch - work.s8 - work.s2);
+    const unsigned long long items = ((unsigned long long)work.s8 / 8 + work.s2 / 2 + work.s1) * (unsigned long long)R;
+    unsigned long long want = (items + warps - 1) / warps;
     if (want < grid) grid = want;
-    kern<<<(unsigned)grid, warps * 32, smem, s>>>(a);
+    kern<<<(unsigned)grid, warps * 32, smem, s>>>(a, work);
     return cudaGetLastError();
 }
 

@@ -111,3 +111,18 @@ def test_wms_training_one_shot_per_lane(code, ckpt, all_iters):
     for a, b in ((w1, w2), (g1, g2)):
         assert np.linalg.norm(b) > 0
         assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("shots", [1, 3, 200, 1601])
+def test_small_code_run_lengths(shots):
+    """The small-code kernel's runs of 8, 2 and 1 shots ([[72]], R = 64: the
+    last 16 shots per resident warp come in short runs): one shot, an odd
+    batch in runs of 1 and 2, a batch with all three."""
+    from paper_2605_14170_gb300 import mbbp
+    H = named_code("bb72").HZ
+    e, _ = oracle.sample(SEED + 2, 0, shots, 72, 0.05, "bsc")
+    s = oracle.syndrome(H, e)
+    llr = channel_llr(72, 0.05).astype(np.float32)
+    B = mbbp.mbbp_build_bases(H, 64, SEED)
+    got = _decode(B, s, llr, 25, 0.625)
+    _assert_exact(got, oracle.mbbp_decode(H, B.sets, s, llr, 25, 0.625, precision="f32"))
