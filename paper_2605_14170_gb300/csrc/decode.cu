@@ -305,9 +305,9 @@ cudaError_t launch_decode_t(const DecodeArgs& a, cudaStream_t s, int sm_count) {
 template <int K, int RULE>
 cudaError_t launch_decode_k(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     // posteriors and the message trace take a kernel of their own, as do
-    // min-sum calls on codes whose rows all fill the kernel width
+    // codes whose rows all fill the kernel width
     if (a.io.c2v || a.io.post) return launch_decode_t<K, RULE, false, true>(a, s, sm_count);
-    if (RULE == MBBP_RULE_NMS && a.B.regular) return launch_decode_t<K, RULE, RULE == MBBP_RULE_NMS, false>(a, s, sm_count);
+    if (a.B.regular) return launch_decode_t<K, RULE, true, false>(a, s, sm_count);
     return launch_decode_t<K, RULE, false, false>(a, s, sm_count);
 }
 

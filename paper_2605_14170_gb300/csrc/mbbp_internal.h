@@ -114,10 +114,11 @@ constexpr int kNumSmallShapes = 3;
 // [[144]], R = 16: with 18, ptxas settles at 96 registers (20 resident warps
 // per SM) and the kernel runs 9% faster than with 8-warp blocks at 116
 // registers (16 warps per SM); tighter budgets (20 or 21 blocks), or 2-warp
-// blocks at 10, were slower.  Four row steps and the sum-product rule need
-// more registers: 16 keeps them unspilled.
+// blocks at 10, were slower.  Four row steps need more registers: 16 keeps
+// them unspilled.  Sum-product, [[144]] R = 16, 4,000 shots at p = 0.04: 16 /
+// 20 / 24 / 28 blocks 2.34 / 2.23 / 2.44 / 2.45 ms.
 __host__ __device__ constexpr int small_min_blocks(int RS, int rule) {
-    return (RS <= 3 && rule == MBBP_RULE_NMS) ? 18 : 16;
+    return rule == MBBP_RULE_SP ? 20 : (RS <= 3 ? 18 : 16);
 }
 
 #ifdef __CUDACC__
