@@ -19,7 +19,9 @@
 // state all measured slower or the same.
 //
 // [[144,12,12]] R = 8, T = 25, checkpoints every 5, batch 4096: forward 0.93 ->
-// 0.74 ms, backward 4.58 -> 2.15 ms; batch 300 R = 4: 0.091 + 0.336 -> 0.084 +
+// 0.72 ms, backward 4.58 -> 1.98 ms (0.74 and 2.15 before the warp's index was
+// broadcast, which lets the compiler keep what depends on it in uniform
+// registers); batch 300 R = 4: 0.091 + 0.336 -> 0.084 +
 // 0.201 ms; [[288,12,18]] R = 4, batch 1500: 0.50 + 2.94 -> 0.38 + 1.04 ms.
 #include <algorithm>
 #include <climits>
@@ -129,7 +131,7 @@ struct Block {
     __device__ __forceinline__ Block(const WmsArgs& args, unsigned char* sm)
         : a(args), L(lanes_layout(DC, args.B.MP, args.B.n)), smem(sm) {
         lane = threadIdx.x & 31;
-        warp = threadIdx.x >> 5;
+        warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);  // known to be uniform
         nw = blockDim.x >> 5;
         slot = lane & (CS - 1);
         sub = lane / CS;
