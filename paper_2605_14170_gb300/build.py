@@ -16,7 +16,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libmbbp.so")
-SOURCES = ["host.cpp", "decode.cu", "decode_small.cu", "decode_serial.cu", "decode_mixed.cu", "wms.cu", "wms_lanes.cu",
+SOURCES = ["host.cpp", "decode.cu", "decode_small.cu", "decode_serial.cu", "decode_serial_lanes.cu", "decode_mixed.cu", "wms.cu", "wms_lanes.cu",
            "aux.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-std=c++20", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall"]

@@ -1,4 +1,6 @@
-// Serial-schedule launches (Section II-B).  Kernel widths 6 and 8 use the
+// Serial-schedule launches (Section II-B).  Batches long enough for it take
+// the one-shot-per-lane kernel (decode_serial_lanes.cu); per-shot LLRs, calls
+// for posteriors, short batches and long codes stay here.  Widths 6 and 8 use the
 // slot path of bp_serial.cuh: a persistent grid whose warps pull shots of
 // one representation at a time from per-representation counters and decode
 // CS of them at once (CS = 4, 2 or 1, the largest that leaves about half of
@@ -84,6 +86,9 @@ cudaError_t launch_width(const DecodeArgs& a, cudaStream_t s, int sm_count) {
 
 cudaError_t launch_decode_serial(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     if (!a.B.edesc || (a.B.DC != 6 && a.B.DC != 8)) return launch_decode_serial_generic(a, s, sm_count);
+    bool taken = false;
+    const cudaError_t e = launch_decode_serial_lanes(a, s, sm_count, &taken);
+    if (e != cudaSuccess || taken) return e;
     const bool reg = a.B.regular != 0;
     if (a.rule == MBBP_RULE_NMS)
         return reg ? launch_width<MBBP_RULE_NMS, true>(a, s, sm_count)

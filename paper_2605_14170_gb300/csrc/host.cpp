@@ -646,6 +646,7 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
     }
     auto slot_of = [&](int pos, int j) { return (pos >> 5) * (32 * K) + 32 * j + (pos & 31); };
     std::vector<uint16_t> lrows16((size_t)R * MP, 0);
+    int lsteps = 0;
     for (int t = 0; t < R; ++t) {
         const RepLayout& L = layouts[t];
         const int M = (int)L.src.size();
@@ -697,6 +698,9 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
         }
         lp[nl] = at;
         B->nlayers[t] = nl;
+        int steps2 = 0;
+        for (int y = 0; y < nl; ++y) steps2 += (lp[y + 1] - lp[y] + 1) / 2;
+        lsteps = std::max(lsteps, steps2);
         if (chunked) {
             // chunk kernel: rows at bank-aware positions, descriptors by position
             const std::vector<int>& sp = L.sp;
@@ -885,6 +889,7 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
     d.edesc = chunked ? reinterpret_cast<const uint4*>(base + o_edesc) : nullptr;
     d.vdesc3 = chunked ? reinterpret_cast<const uint4*>(base + o_vdesc3) : nullptr;
     d.lpos = chunked ? reinterpret_cast<const uint16_t*>(base + o_lpos) : nullptr;
+    d.lsteps = lsteps;
     d.rinfo_s = chunked ? reinterpret_cast<const uint32_t*>(base + o_rinfo_s) : nullptr;
     *out = B;
     return MBBP_OK;

@@ -64,6 +64,7 @@ struct DevBases {
     // positions in layer order, and per position src row | degree << 16
     const uint16_t* lpos;     // [R][MP]
     const uint32_t* rinfo_s;  // [R][MP]
+    int lsteps;               // most two-row steps of a representation, its layers padded to whole steps
 };
 
 // Shared memory of one warp of the serial chunk kernel (bp_serial.cuh) for
@@ -274,6 +275,9 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t s, int sm_count);
 cudaError_t launch_decode_serial(const DecodeArgs& a, cudaStream_t s, int sm_count);
 cudaError_t launch_decode_serial_generic(const DecodeArgs& a, cudaStream_t s, int sm_count);
 cudaError_t launch_decode_small(const DecodeArgs& a, cudaStream_t s, int sm_count);
+// One shot per lane (decode_serial_lanes.cu); *taken = false, nothing launched,
+// for calls that stay with the warp-per-slot kernel.
+cudaError_t launch_decode_serial_lanes(const DecodeArgs& a, cudaStream_t s, int sm_count, bool* taken);
 cudaError_t launch_fws(const FwsArgs& a, cudaStream_t s);
 // Device address of the fixed scratch array on the current device (looked up
 // on the first call per device).

@@ -126,3 +126,32 @@ def test_small_code_run_lengths(shots):
     B = mbbp.mbbp_build_bases(H, 64, SEED)
     got = _decode(B, s, llr, 25, 0.625)
     _assert_exact(got, oracle.mbbp_decode(H, B.sets, s, llr, 25, 0.625, precision="f32"))
+
+
+@pytest.mark.parametrize("rule", ["nms", "sp"])
+@pytest.mark.parametrize("code,R,shots", [("bb72", 64, 2000), ("irregular", 64, 2003), ("gb90w4", 20, 1001),
+                                          ("gb166", 8, 1300)])
+def test_serial_one_shot_per_lane(code, R, shots, rule):
+    """Serial batches long enough for the one-shot-per-lane kernel: slots
+    refilled several times, odd layers and variable classes, rows that do not
+    fill the width, both widths, zero syndromes among the shots.  Min-sum
+    against the FP32 oracle bit for bit; both rules against the warp-per-slot
+    kernel (which the same LLRs given per shot take) bit for bit."""
+    from paper_2605_14170_gb300 import mbbp
+    H = named_code("bb72").HZ if code == "bb72" else CODES[code]()
+    n = H.shape[1]
+    e, _ = oracle.sample(SEED + 3, 0, shots, n, 0.04, "bsc")
+    s = oracle.syndrome(H, e)
+    s[::7] = 0
+    rng = np.random.default_rng(9)
+    llr = rng.uniform(1.0, 4.0, n).astype(np.float32)
+    llr[::11] = -0.5
+    B = mbbp.mbbp_build_bases(H, R, SEED)
+    kw = dict(rule=mbbp.RULE_SP if rule == "sp" else mbbp.RULE_NMS, schedule=mbbp.SCHEDULE_SERIAL)
+    got = _decode(B, s, llr, 12, 0.8, **kw)
+    ref = _decode(B, s, np.tile(llr, (shots, 1)), 12, 0.8, **kw)
+    for key in ("conv", "iters", "cand", "selected", "success", "e_hat"):
+        assert np.array_equal(got[key], ref[key]), key
+    if rule == "nms":
+        _assert_exact(got, oracle.mbbp_decode(H, B.sets, s, llr, 12, 0.8, precision="f32",
+                                              schedule=oracle.SCHEDULE_SERIAL))
