@@ -40,7 +40,7 @@ decode_kernel(const DecodeArgs a) {
     __shared__ unsigned long long group_item[MAXW];
     const DevBases& B = a.B;
     const int lane = threadIdx.x & 31;
-    const int grp = (int)(threadIdx.x >> 5) / G;
+    const int grp = warp_index() / G;
     const int gt = (int)(threadIdx.x % (32 * G));
     const int bar = 1 + grp;
     const generic_bp::WarpLayout L = generic_bp::warp_layout(DC, B.MP, B.mpad, B.n);
@@ -62,7 +62,7 @@ decode_kernel(const DecodeArgs a) {
             // only after the item's last barrier, which every reader passed
             if (gt == 0) group_item[grp] = atomicAdd(a.counter, 1ull);
             generic_bp::gsync<G>(bar);
-            item = group_item[grp];
+            item = __shfl_sync(kFull, group_item[grp], 0);
         }
         if (item >= a.total_items) break;
         const int b = (int)(item / batch);
@@ -79,7 +79,7 @@ decode_serial_kernel(const DecodeArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const DevBases& B = a.B;
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index();
     const int R = B.R;
     const generic_bp::WarpLayout L = generic_bp::warp_layout(DC, B.MP, B.mpad, B.n);
     const int per_warp = generic_bp::serial_warp_bytes(DC, B.MP, B.mpad, B.n);

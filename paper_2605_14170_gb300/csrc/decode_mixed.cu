@@ -51,7 +51,7 @@ template <int RULE, int VS, int RS, int ORS>
 __global__ void __launch_bounds__(32, small_min_blocks(RS, RULE)) mixed_small_kernel(const MixedArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     char* smc = reinterpret_cast<char*>(smem);
-    const uint32_t wbase = (uint32_t)(threadIdx.x >> 5) * a.warp_bytes;
+    const uint32_t wbase = 0;  // one warp per block
     MixedItem it;
     while (next_item(a, it)) {
         const MixedCode& mc = a.codes[it.c];
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(32, small_min_blocks(RS, RULE)) mixed_small_ke
 template <int RULE>
 __global__ void __launch_bounds__(kMixedMaxWarps * 32) mixed_generic_kernel(const MixedArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const uint32_t wbase = (uint32_t)(threadIdx.x >> 5) * a.warp_bytes;
+    const uint32_t wbase = (uint32_t)warp_index() * a.warp_bytes;
     MixedItem it;
     while (next_item(a, it)) {
         const MixedCode& mc = a.codes[it.c];

@@ -21,7 +21,7 @@ __global__ void __launch_bounds__(kSerialWarps * 32, kSerialMinBlocks)
 decode_serial_chunk_kernel(const DecodeArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const DevBases& B = a.B;
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index();
     const int R = B.R;
     const int hcol_bytes = generic_bp::align16(DC * B.mpad * 2);
     const serial_bp::Layout L = serial_bp::layout(DC, B.MP, B.n, CS);

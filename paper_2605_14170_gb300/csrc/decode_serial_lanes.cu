@@ -128,8 +128,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) decode_serial_lanes_kernel(con
     const SerialLanesLayout L = serial_lanes_layout(DC, B.lsteps, m, n);
     const int lane = threadIdx.x & 31, slot = lane % kShots, sub = lane / kShots;
     const int nw = (int)(blockDim.x >> 5) / kGroups;  // warps of a group
-    // broadcast, so that what depends on the warp is known to be uniform
-    const int wid = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);
+    const int wid = warp_index();
     const int grp = wid / nw, warp = wid - grp * nw;
     const int gthreads = nw * 32, gt = warp * 32 + lane, bar = 1 + grp;
     unsigned char* area = smem + L.group0 + grp * L.group_bytes;

@@ -34,7 +34,7 @@ decode_small_kernel(const DecodeArgs a, const SmallWork work) {
     extern __shared__ __align__(16) float smsg[];
     const DevBases& B = a.B;
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
+    const int warp = kSmallWarps == 1 ? 0 : warp_index();
     const unsigned R = (unsigned)B.R;
     char* smc = reinterpret_cast<char*>(smsg);
     const uint32_t wbase = (uint32_t)(warp * small_bp::warp_floats(B.MP, VS, ORS) * 4);

@@ -123,6 +123,11 @@ __host__ __device__ constexpr int small_min_blocks(int RS, int rule) {
 }
 
 #ifdef __CUDACC__
+// The warp's index in its block, broadcast so that the compiler knows that
+// what depends on it (a warp's shared-memory area, loop bounds, branches) is
+// uniform and can keep it in uniform registers.
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 // min(|a|, |b|) with the sign sign(a) XOR sign(b), one instruction at the rate
 // of a plain min: folded over a row's edges it yields the excluded minimum
 // and the sign product of Eq. (2) together.  A NaN operand loses to a number

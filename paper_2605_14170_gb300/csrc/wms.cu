@@ -215,7 +215,7 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
     const DevBases& B = a.B;
     const int lane = (int)(threadIdx.x % GT);  // the thread's index in its group
     const int wig = lane >> 5;                  // the warp's index in its group
-    const int grp = (int)(threadIdx.x >> 5) / G;
+    const int grp = warp_index() / G;
     const int bar = 1 + grp;
     const int MP = B.MP, n = B.n, m_rows = B.m, R = B.R, W = B.W;
     const WmsLayout L = wms_layout(DC, MP, n, a.ckpt);
@@ -244,7 +244,7 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
             // rewritten only after the item's last barrier, which every reader passed
             if (lane == 0) group_item[grp] = atomicAdd(a.counter, 1ull);
             generic_bp::gsync<G>(bar);
-            g = group_item[grp];
+            g = __shfl_sync(kFull, group_item[grp], 0);
         }
         if (g >= a.total_items) break;
         const int b = (int)(g / batch);
@@ -391,7 +391,7 @@ wms_backward_kernel(const WmsArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const DevBases& B = a.B;
     const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
+    const int warp = warp_index();
     const int MP = B.MP, n = B.n, m_rows = B.m, R = B.R;
     const WmsLayout L = wms_layout(DC, MP, n, a.ckpt);
     const size_t gwarp = (size_t)blockIdx.x * (blockDim.x >> 5) + warp;

@@ -131,7 +131,7 @@ struct Block {
     __device__ __forceinline__ Block(const WmsArgs& args, unsigned char* sm)
         : a(args), L(lanes_layout(DC, args.B.MP, args.B.n)), smem(sm) {
         lane = threadIdx.x & 31;
-        warp = __shfl_sync(kFull, (int)(threadIdx.x >> 5), 0);  // known to be uniform
+        warp = warp_index();
         nw = blockDim.x >> 5;
         slot = lane & (CS - 1);
         sub = lane / CS;
