@@ -113,7 +113,7 @@ __device__ __forceinline__ void wms_var_pass(const DevBases& B, int b, const uin
             const uint4 d = dn;
             if (p + GT < n) dn = __ldg(vd6 + p + GT);
             const int v = d.x & 0xffff, deg = (int)(d.x >> 16);
-            const float pv = wms_var_dispatch(deg, m, q, d, mu[v]);
+            const float pv = wms_var_dispatch(deg, m, q, d, mu[p]);
             if (post) post[v] = pv;
         }
         return;
@@ -132,7 +132,7 @@ __device__ __forceinline__ void wms_var_pass(const DevBases& B, int b, const uin
             mv[i] = (i < deg) ? m[s[i]] : 0.0f;
         }
         float P[DV + 1];  // prefix sums, as in the packed branch
-        P[0] = mu[v];
+        P[0] = mu[p];
 #pragma unroll
         for (int i = 0; i < DV; ++i) P[i + 1] = (i < deg) ? __fadd_rn(P[i], mv[i]) : P[i];
         if (post) post[v] = P[DV];
@@ -221,8 +221,8 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
     const WmsLayout L = wms_layout(DC, MP, n, a.ckpt);
     float* m = reinterpret_cast<float*>(smem + grp * L.fwd_bytes);
     float* q = m + L.S;
-    float* mu = q + L.S;
-    float* post = mu + L.npad;  // post[n] = +0: the padding column of hcol
+    float* mu = q + L.S;        // by position in vdesc order
+    float* post = mu + L.npad;  // by variable; post[n] = +0: the padding column of hcol
     const int orow_steps = (B.mpad + GT - 1) / GT;
     const int row_steps = (MP + GT - 1) / GT;
     // H's columns for the halting test, once per block
@@ -257,7 +257,6 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
         const uint8_t* sy = a.synd + (size_t)shot * m_rows;
         for (int v = lane; v < n; v += GT) {
             const float x = __fadd_rn(__ldg(llr + v), 0.0f);  // -0 -> +0 (sign bits decide the check rule)
-            mu[v] = x;
             post[v] = x;
         }
         if (lane == 0) post[n] = 0.0f;
@@ -275,7 +274,8 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
         for (int p = lane; p < n; p += GT) {  // q^(0) = mu
             const uint2 d = __ldg(vd + p);
             const int v = d.y & 0xffff, deg = (int)(d.y >> 16);
-            for (int i = 0; i < deg; ++i) q[__ldg(B.vslot + d.x + i)] = mu[v];
+            mu[p] = post[v];
+            for (int i = 0; i < deg; ++i) q[__ldg(B.vslot + d.x + i)] = mu[p];
         }
         generic_bp::gsync<G>(bar);
         int K = 0;
@@ -416,7 +416,8 @@ wms_backward_kernel(const WmsArgs a) {
         const int Mb = __ldg(B.rows + b);
         const float* llr = a.llr + (size_t)shot * a.llr_stride;
         const uint8_t* sy = a.synd + (size_t)shot * m_rows;
-        for (int v = lane; v < n; v += 32) mu[v] = __fadd_rn(__ldg(llr + v), 0.0f);  // as the forward pass
+        for (int p = lane; p < n; p += 32)  // as the forward pass, by position
+            mu[p] = __fadd_rn(__ldg(llr + (__ldg(&vd[p].y) & 0xffffu)), 0.0f);
         uint32_t sb = 0;
         for (int k = 0; k < (MP >> 5); ++k) {
             const int r = lane + 32 * k;
@@ -456,7 +457,7 @@ wms_backward_kernel(const WmsArgs a) {
                     for (int p = lane; p < n; p += 32) {
                         const uint2 d = __ldg(vd + p);
                         const int v = d.y & 0xffff, deg = (int)(d.y >> 16);
-                        for (int i = 0; i < deg; ++i) q[__ldg(B.vslot + d.x + i)] = mu[v];
+                        for (int i = 0; i < deg; ++i) q[__ldg(B.vslot + d.x + i)] = mu[p];
                     }
                 } else {
                     wms_var_pass<DV>(B, b, vd, mprev, q, mu, nullptr);
@@ -475,7 +476,7 @@ wms_backward_kernel(const WmsArgs a) {
                     for (int p = lane; p < n; p += 32) {
                         const uint2 d = __ldg(vd + p);
                         const int v = d.y & 0xffff, deg = (int)(d.y >> 16);
-                        for (int i = 0; i < deg; ++i) q[__ldg(B.vslot + d.x + i)] = mu[v];
+                        for (int i = 0; i < deg; ++i) q[__ldg(B.vslot + d.x + i)] = mu[p];
                     }
                 } else {
                     wms_var_pass<DV>(B, b, vd, mprev, q, mu, nullptr);
@@ -569,7 +570,7 @@ wms_backward_kernel(const WmsArgs a) {
                             if (i < deg) G += generic_bp::msg_at(gq, o[i]);
                         float gp = 0.0f;
                         if (a.all_iters) {
-                            float acc = mu[v];
+                            float acc = mu[p];
 #pragma unroll
                             for (int i = 0; i < 6; ++i)
                                 if (i < deg) acc = __fadd_rn(acc, generic_bp::msg_at(const_cast<float*>(mprev), o[i]));
@@ -590,7 +591,7 @@ wms_backward_kernel(const WmsArgs a) {
                         // all_iters: the BCE of post^(t-1) joins dL/dm^(t-1)
                         float gp = 0.0f;
                         if (a.all_iters) {
-                            float acc = mu[v];
+                            float acc = mu[p];
                             for (int i = 0; i < deg; ++i) acc = __fadd_rn(acc, mprev[__ldg(sl + i)]);
                             const uint32_t ev = (__ldg(a.etrue + (size_t)shot * B.W + (v >> 5)) >> (v & 31)) & 1u;
                             gp = lw * ((float)ev - 1.0f / (1.0f + expf(acc)));
