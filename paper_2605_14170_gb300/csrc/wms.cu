@@ -206,7 +206,7 @@ __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const u
 // mu, and mu enters as llr + 0).  The arguments come by value (taken by
 // reference from the kernel's parameter, the decode on a length-882 code
 // measured 5% slower).
-template <int DC, int DV, int G>
+template <int DC, int DV, int G, bool DEC>
 __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long group_item[kWmsWarps];
@@ -227,7 +227,7 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
     const int row_steps = (MP + GT - 1) / GT;
     // H's columns for the halting test, once per block
     uint16_t* hcol_s = reinterpret_cast<uint16_t*>(smem + (blockDim.x / GT) * L.fwd_bytes);
-    if (a.decode) {
+    if (DEC) {
         for (int i = threadIdx.x; i < DC * B.mpad; i += blockDim.x) hcol_s[i] = __ldg(B.hcol + i);
         __syncthreads();
     }
@@ -266,7 +266,7 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
             const int r = lane + GT * k;
             if (r < Mb) sb |= (uint32_t)(__ldg(sy + (__ldg(rinfo + r) & 0xffffu)) & 1u) << k;
         }
-        for (int k = 0; a.decode && k < orow_steps; ++k) {
+        for (int k = 0; DEC && k < orow_steps; ++k) {
             const int r = lane + GT * k;
             if (r < m_rows) sbo |= (uint32_t)(__ldg(sy + r) & 1u) << k;
         }
@@ -281,9 +281,9 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
         int K = 0;
         bool conv = false;
         float lacc = 0.f;  // this lane's BCE of the posteriors of iterations 1..T-1 (all_iters)
-        const int iters = a.decode ? a.iters : a.T;
+        const int iters = DEC ? a.iters : a.T;
         for (int it = 0;; ++it) {
-            if (a.decode) {
+            if (DEC) {
                 // the first row group decides most unconverged iterations,
                 // so the other groups are tested only if it passed
                 bool ok = true;
@@ -308,7 +308,7 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
                 break;
             }
             const int tp = min(it, a.T - 1);  // iterations past T reuse the last weights
-            if (a.wg) {
+            if (DEC) {
                 const float2* wgt = a.wg + ((size_t)b * a.T + tp) * DC * MP;
                 wms_check_pass<DC, G, true>(B, b, rinfo, Mb, sb, q, m, reinterpret_cast<const float*>(wgt),
                                             nullptr);
@@ -320,7 +320,7 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
             generic_bp::gsync<G>(bar);
             wms_var_pass<DV, G>(B, b, vd, m, q, mu, post);
             generic_bp::gsync<G>(bar);
-            if (!a.decode) {
+            if (!DEC) {
                 if (a.ckpt_buf && (it + 1) % a.ckpt == 0 && it + 1 < a.T) {
                     float* dst = a.ckpt_buf + ((size_t)item * a.nckpt + ((it + 1) / a.ckpt - 1)) * L.S;
                     for (int i = lane; i < L.S; i += GT) dst[i] = m[i];
@@ -331,9 +331,9 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
                 }
             }
         }
-        if (a.post)
+        if (!DEC && a.post)
             for (int v = lane; v < n; v += GT) a.post[item * n + v] = post[v];
-        if (a.decode) {
+        if (DEC) {
             // warp wig packs the candidate words wig, wig + G, ...
             const int wl = lane & 31;
             for (int w = wig; w < W; w += G) {
@@ -365,18 +365,22 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
     }
 }
 
-// One warp per item: the compiler's own register choice.
-template <int DC, int DV>
+// DEC: decode (halting rule, candidates), else the training forward.  Compiled
+// apart, since either one carried the other's tests and registers: decode on
+// [[288,12,18]] R = 8, 2,060 shots 548 -> 299 us, on the length-882 code R = 64,
+// 2,000 shots 7.16 -> 6.99 ms.  One warp per item: the compiler's own register
+// choice.
+template <int DC, int DV, bool DEC>
 __global__ void __launch_bounds__(kWmsWarps * 32) wms_forward_warp_kernel(const WmsArgs a) {
-    wms_forward_items<DC, DV, 1>(a);
+    wms_forward_items<DC, DV, 1, DEC>(a);
 }
 
 // G > 1 warps per item: registers for three 8-warp blocks per SM, the
 // residency that the message areas allow for the codes that take G > 1
 // (without the bound the compiler stops at 64 registers and spills).
-template <int DC, int DV, int G>
+template <int DC, int DV, int G, bool DEC>
 __global__ void __launch_bounds__(kWmsWarps * 32, 3) wms_forward_kernel(const WmsArgs a) {
-    wms_forward_items<DC, DV, G>(a);
+    wms_forward_items<DC, DV, G, DEC>(a);
 }
 
 // SMEM_ST: the segment's recomputed states sit in shared memory after the
@@ -649,7 +653,7 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ gra
     p[i] = fminf(fmaxf(x, lo), hi);
 }
 
-template <int K, int G>
+template <int K, int G, bool DEC>
 cudaError_t launch_forward_g(const WmsArgs& a, size_t fixed, size_t per_item, int warps, int per_sm,
                              cudaStream_t s, int sm_count) {
     const unsigned long long groups = (unsigned long long)(warps / G);
@@ -658,50 +662,54 @@ cudaError_t launch_forward_g(const WmsArgs& a, size_t fixed, size_t per_item, in
     unsigned long long grid = (unsigned long long)per_sm * sm_count;
     if (want < grid) grid = want;
     if constexpr (G == 1)
-        wms_forward_warp_kernel<K, K><<<(unsigned)grid, warps * 32, smem, s>>>(a);
+        wms_forward_warp_kernel<K, K, DEC><<<(unsigned)grid, warps * 32, smem, s>>>(a);
     else
-        wms_forward_kernel<K, K, G><<<(unsigned)grid, warps * 32, smem, s>>>(a);
+        wms_forward_kernel<K, K, G, DEC><<<(unsigned)grid, warps * 32, smem, s>>>(a);
     return cudaGetLastError();
+}
+
+// forward / decode: G warps per item, G in {1, 2, 4}; per G the block size (a
+// multiple of G, up to 8 warps) with the most resident warps per SM within 200
+// KB of shared memory per block (for the decode H's columns once, then one area
+// per item); a larger G only when it holds at least half again as many warps
+// as the best smaller one
+template <int K, bool DEC>
+cudaError_t launch_forward(const WmsArgs& a, cudaStream_t s, int sm_count) {
+    const WmsLayout L = wms_layout(K, a.B.MP, a.B.n, a.ckpt);
+    if (L.fwd_bytes > 200 * 1024) return cudaErrorInvalidConfiguration;
+    const size_t fixed = (size_t)((K * a.B.mpad * 2 + 15) & ~15);
+    const void* kerns[3] = {reinterpret_cast<const void*>(wms_forward_warp_kernel<K, K, DEC>),
+                            reinterpret_cast<const void*>(wms_forward_kernel<K, K, 2, DEC>),
+                            reinterpret_cast<const void*>(wms_forward_kernel<K, K, 4, DEC>)};
+    int best_g = -1, best_w = 0, best_b = 0;
+    for (int gi = 0; gi < 3; ++gi) {
+        const int G = 1 << gi;
+        int warps = 0, per_sm = 0;
+        for (int w = G; w <= kWmsWarps && fixed + (size_t)(w / G) * L.fwd_bytes <= 200 * 1024; w += G) {
+            int b = 0;
+            cudaError_t e = prepare_kernel(kerns[gi], w * 32, fixed + (size_t)(w / G) * L.fwd_bytes, &b);
+            if (e != cudaSuccess) return e;
+            if (b * w > per_sm * warps) {
+                warps = w;
+                per_sm = b;
+            }
+        }
+        if (warps > 0 && (best_g < 0 || 2 * warps * per_sm >= 3 * best_w * best_b)) {
+            best_g = gi;
+            best_w = warps;
+            best_b = per_sm;
+        }
+    }
+    if (best_g < 0) return cudaErrorInvalidConfiguration;
+    if (best_g == 0) return launch_forward_g<K, 1, DEC>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
+    if (best_g == 1) return launch_forward_g<K, 2, DEC>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
+    return launch_forward_g<K, 4, DEC>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
 }
 
 template <int K>
 cudaError_t launch_wms_t(const WmsArgs& a, bool backward, cudaStream_t s, int sm_count) {
+    if (!backward) return a.decode ? launch_forward<K, true>(a, s, sm_count) : launch_forward<K, false>(a, s, sm_count);
     const WmsLayout L = wms_layout(K, a.B.MP, a.B.n, a.ckpt);
-    if (!backward) {
-        // forward / decode: G warps per item, G in {1, 2, 4}; per G the block
-        // size (a multiple of G, up to 8 warps) with the most resident warps
-        // per SM within 200 KB of shared memory per block (H's columns once,
-        // then one area per item); a larger G only when it holds at least
-        // half again as many warps as the best smaller one
-        if (L.fwd_bytes > 200 * 1024) return cudaErrorInvalidConfiguration;
-        const size_t fixed = (size_t)((K * a.B.mpad * 2 + 15) & ~15);
-        const void* kerns[3] = {reinterpret_cast<const void*>(wms_forward_warp_kernel<K, K>),
-                                reinterpret_cast<const void*>(wms_forward_kernel<K, K, 2>),
-                                reinterpret_cast<const void*>(wms_forward_kernel<K, K, 4>)};
-        int best_g = -1, best_w = 0, best_b = 0;
-        for (int gi = 0; gi < 3; ++gi) {
-            const int G = 1 << gi;
-            int warps = 0, per_sm = 0;
-            for (int w = G; w <= kWmsWarps && fixed + (size_t)(w / G) * L.fwd_bytes <= 200 * 1024; w += G) {
-                int b = 0;
-                cudaError_t e = prepare_kernel(kerns[gi], w * 32, fixed + (size_t)(w / G) * L.fwd_bytes, &b);
-                if (e != cudaSuccess) return e;
-                if (b * w > per_sm * warps) {
-                    warps = w;
-                    per_sm = b;
-                }
-            }
-            if (warps > 0 && (best_g < 0 || 2 * warps * per_sm >= 3 * best_w * best_b)) {
-                best_g = gi;
-                best_w = warps;
-                best_b = per_sm;
-            }
-        }
-        if (best_g < 0) return cudaErrorInvalidConfiguration;
-        if (best_g == 0) return launch_forward_g<K, 1>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
-        if (best_g == 1) return launch_forward_g<K, 2>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
-        return launch_forward_g<K, 4>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
-    }
     const size_t st_bytes = (size_t)a.ckpt * L.S * 4;
     const bool smem_st = wms_states_in_smem(a.B, a.ckpt);
     const size_t per_warp = L.bwd_bytes + (smem_st ? st_bytes : 0);
