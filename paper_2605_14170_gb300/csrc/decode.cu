@@ -164,6 +164,69 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32) fws_kernel(const FwsArgs 
     }
 }
 
+// FWS for R <= 32 candidates of at most WM words: GL = 2^LR >= R lanes per shot,
+// a candidate per lane in registers.  Equal candidates are found with a match
+// over the lanes word by word, so a shot costs W matches instead of R
+// comparisons of W words; counts and weights are small enough for 32-bit
+// products (count <= 32, weight <= 32 WM).  Bound by issue slots and the
+// candidates' loads: [[144,12,12]] R = 16, 200,000 shots 248 -> 35 us.
+template <int LR, int WM>
+__global__ void __launch_bounds__(kWarpsPerBlock * 32) fws_lanes_kernel(const FwsArgs a) {
+    constexpr int GL = 1 << LR;
+    const int lane = threadIdx.x & 31, r = lane & (GL - 1), base = lane & ~(GL - 1);
+    const long long first = ((long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5)) * (32 / GL);
+    if (first >= a.batch) return;  // uniform per warp
+    const int R = a.R, W = a.W, n = a.n;
+    const int shot = (int)min(first + lane / GL, (long long)a.batch - 1);  // past the end: the last shot again
+    const uint32_t* src = a.cand + (size_t)shot * R * W;
+    const bool conv = r < R && __ldg(a.conv + (size_t)shot * R + r) != 0;
+    uint32_t eq = __ballot_sync(kFull, conv) & (GL == 32 ? kFull : (((1u << (GL & 31)) - 1u) << base));
+    int weight = 0;
+#pragma unroll
+    for (int k = 0; k < WM; ++k) {
+        if (k < W) {
+            const uint32_t c = r < R ? __ldg(src + (size_t)r * W + k) : 0u;
+            weight += __popc(c);
+            eq &= __match_any_sync(kFull, c);
+        }
+    }
+    // count << 21 | weight << 6 | index; 0 for a candidate that did not converge
+    uint32_t best = conv ? ((uint32_t)__popc(eq) << 21) | ((uint32_t)weight << 6) | (uint32_t)r : 0u;
+#pragma unroll
+    for (int off = GL / 2; off > 0; off >>= 1) {
+        const uint32_t o = __shfl_xor_sync(kFull, best, off);
+        const uint32_t lhs = (o >> 21) * (((best >> 6) & 0x7fffu) + 1u), rhs = (best >> 21) * (((o >> 6) & 0x7fffu) + 1u);
+        if (lhs > rhs || (lhs == rhs && (o & 63u) < (best & 63u))) best = o;
+    }
+    const int sel = (best >> 21) ? (int)(best & 63u) : -1;
+    if (first + lane / GL >= a.batch) return;
+    uint8_t* out = a.e_hat + (size_t)shot * n;
+    const uint32_t* words = src + (size_t)max(sel, 0) * W;
+    if ((n & 3) == 0 && (reinterpret_cast<uintptr_t>(a.e_hat) & 3) == 0) {
+        // four bytes at a time: bit i of the nibble to byte i
+        for (int t = r; 4 * t < n; t += GL) {
+            const uint32_t nib = sel >= 0 ? (__ldg(words + (t >> 3)) >> (4 * (t & 7))) & 15u : 0u;
+            reinterpret_cast<uint32_t*>(out)[t] = (nib * 0x00204081u) & 0x01010101u;
+        }
+    } else {
+        for (int v = r; v < n; v += GL) out[v] = sel >= 0 ? (uint8_t)((__ldg(words + (v >> 5)) >> (v & 31)) & 1u) : 0;
+    }
+    if (r == 0) {
+        a.success[shot] = sel >= 0 ? 1 : 0;
+        if (a.selected) a.selected[shot] = (int16_t)sel;
+    }
+}
+
+constexpr int kFwsWords = 10;  // candidates up to 320 variables stay in registers
+
+template <int LR>
+cudaError_t launch_fws_lanes(const FwsArgs& a, cudaStream_t s) {
+    constexpr int shots = kWarpsPerBlock * (32 >> LR);
+    const unsigned grid = (unsigned)(((long long)a.batch + shots - 1) / shots);
+    fws_lanes_kernel<LR, kFwsWords><<<grid, kWarpsPerBlock * 32, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 // One warp per shot: the least-metric selector over the R candidates
 // (R <= 64).  The metric of candidate a is the float sum, in ascending
 // variable order, of the shot's LLRs over the set bits of a; the smallest
@@ -402,6 +465,12 @@ cudaError_t launch_fws(const FwsArgs& a, cudaStream_t s) {
         const unsigned grid = (unsigned)((a.batch + warps - 1) / warps);
         lms_kernel<<<grid, warps * 32, 0, s>>>(a);
         return cudaGetLastError();
+    }
+    if (a.R <= 32 && a.W <= kFwsWords) {
+        if (a.R <= 4) return launch_fws_lanes<2>(a, s);
+        if (a.R <= 8) return launch_fws_lanes<3>(a, s);
+        if (a.R <= 16) return launch_fws_lanes<4>(a, s);
+        return launch_fws_lanes<5>(a, s);
     }
     const size_t per_warp = (size_t)a.R * a.W * 4;
     int warps = kWarpsPerBlock;
