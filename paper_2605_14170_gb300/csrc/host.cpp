@@ -39,7 +39,7 @@ struct mbbp_plan {
 };
 
 struct mbbp_logicals {
-    int m = 0, n = 0, k = 0, K = 0, mpad = 0, W = 0, device = 0;
+    int m = 0, n = 0, k = 0, K = 0, mpad = 0, W = 0, device = 0, sm_count = 0;
     std::vector<uint8_t> ops;  // k x n
     void* dmem = nullptr;
     DevLogicals dev{};
@@ -1069,7 +1069,7 @@ mbbp_status mbbp_syndrome(const mbbp_bases* B, int batch, const uint32_t* e, uin
     if (batch == 0) return MBBP_OK;
     if (!e || !s) return fail(MBBP_E_INVALID, "mbbp_syndrome: NULL buffer");
     if (mbbp_status st = check_device(B->device)) return st;
-    cudaError_t err = launch_syndrome(B->dev, batch, e, s, (cudaStream_t)stream);
+    cudaError_t err = launch_syndrome(B->dev, batch, e, s, (cudaStream_t)stream, B->sm_count);
     return err == cudaSuccess ? MBBP_OK : cuda_fail(err, "mbbp_syndrome");
 }
 
@@ -1737,13 +1737,21 @@ mbbp_status mbbp_logicals_build(const uint8_t* H, int m, const uint8_t* H_other,
     std::vector<uint16_t> hcol((size_t)K * L->mpad, (uint16_t)n);
     for (int r = 0; r < m; ++r)
         for (int j = 0; j < (int)g.rcols[r].size(); ++j) hcol[(size_t)j * L->mpad + r] = (uint16_t)g.rcols[r][j];
+    std::vector<uint32_t> hmask((size_t)m * L->W, 0);
+    for (int r = 0; r < m; ++r)
+        for (int c : g.rcols[r]) hmask[(size_t)r * L->W + (c >> 5)] |= 1u << (c & 31);
     const size_t o_l = align256(hcol.size() * 2);
-    const size_t total = o_l + align256(lmask.size() * 4);
+    const size_t o_h = o_l + align256(lmask.size() * 4);
+    const size_t total = o_h + align256(hmask.size() * 4);
     cudaError_t e = cudaGetDevice(&L->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&L->sm_count, cudaDevAttrMultiProcessorCount, L->device);
     if (e == cudaSuccess) e = cudaMalloc(&L->dmem, total);
     if (e == cudaSuccess) e = cudaMemcpy(L->dmem, hcol.data(), hcol.size() * 2, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(static_cast<char*>(L->dmem) + o_l, lmask.data(), lmask.size() * 4,
+                       cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(static_cast<char*>(L->dmem) + o_h, hmask.data(), hmask.size() * 4,
                        cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         if (L->dmem) cudaFree(L->dmem);
@@ -1752,6 +1760,7 @@ mbbp_status mbbp_logicals_build(const uint8_t* H, int m, const uint8_t* H_other,
     }
     L->dev.hcol = static_cast<const uint16_t*>(L->dmem);
     L->dev.lmask = reinterpret_cast<const uint32_t*>(static_cast<char*>(L->dmem) + o_l);
+    L->dev.hmask = reinterpret_cast<const uint32_t*>(static_cast<char*>(L->dmem) + o_h);
     L->dev.m = m; L->dev.n = n; L->dev.k = k; L->dev.DC = K; L->dev.mpad = L->mpad; L->dev.W = L->W;
     *out = L;
     return MBBP_OK;
@@ -1777,7 +1786,7 @@ mbbp_status mbbp_judge(const mbbp_logicals* L, int batch, const uint32_t* e, con
     if (batch == 0) return MBBP_OK;
     if (!e || !e_hat) return fail(MBBP_E_INVALID, "mbbp_judge: NULL buffer");
     if (mbbp_status st = check_device(L->device)) return st;
-    cudaError_t err = launch_judge(L->dev, batch, e, e_hat, fail_out, counts, (cudaStream_t)stream);
+    cudaError_t err = launch_judge(L->dev, batch, e, e_hat, fail_out, counts, (cudaStream_t)stream, L->sm_count);
     return err == cudaSuccess ? MBBP_OK : cuda_fail(err, "mbbp_judge");
 }
 

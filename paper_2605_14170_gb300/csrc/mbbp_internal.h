@@ -202,6 +202,7 @@ struct FwsArgs {
 struct DevLogicals {
     const uint16_t* hcol;     // [DC][mpad]
     const uint32_t* lmask;    // [k][W]
+    const uint32_t* hmask;    // [m][W] rows of H as bit masks
     int m, n, k, DC, mpad, W;
 };
 
@@ -296,9 +297,9 @@ cudaError_t launch_probe(int kind, int rounds, float* sink, cudaStream_t s, doub
 cudaError_t launch_sample(int n, int batch, uint64_t first_shot, uint64_t seed, uint64_t T,
                           int noise, uint32_t* ex, uint32_t* ez, cudaStream_t s);
 cudaError_t launch_syndrome(const DevBases& B, int batch, const uint32_t* e, uint8_t* synd,
-                            cudaStream_t s);
+                            cudaStream_t s, int sm_count);
 cudaError_t launch_judge(const DevLogicals& L, int batch, const uint32_t* e,
                          const uint8_t* e_hat, uint8_t* fail, unsigned long long* counts,
-                         cudaStream_t s);
+                         cudaStream_t s, int sm_count);
 
 }  // namespace mbbp

@@ -460,7 +460,7 @@ wms_backward_kernel(const WmsArgs a) {
                 if (t - 1 == 0) {
                     for (int p = lane; p < n; p += 32) {
                         const uint2 d = __ldg(vd + p);
-                        const int v = d.y & 0xffff, deg = (int)(d.y >> 16);
+                        const int deg = (int)(d.y >> 16);
                         for (int i = 0; i < deg; ++i) q[__ldg(B.vslot + d.x + i)] = mu[p];
                     }
                 } else {
@@ -479,7 +479,7 @@ wms_backward_kernel(const WmsArgs a) {
                 if (t - 1 == 0) {
                     for (int p = lane; p < n; p += 32) {
                         const uint2 d = __ldg(vd + p);
-                        const int v = d.y & 0xffff, deg = (int)(d.y >> 16);
+                        const int deg = (int)(d.y >> 16);
                         for (int i = 0; i < deg; ++i) q[__ldg(B.vslot + d.x + i)] = mu[p];
                     }
                 } else {

@@ -155,3 +155,60 @@ def test_serial_one_shot_per_lane(code, R, shots, rule):
     if rule == "nms":
         _assert_exact(got, oracle.mbbp_decode(H, B.sets, s, llr, 12, 0.8, precision="f32",
                                               schedule=oracle.SCHEDULE_SERIAL))
+
+
+@pytest.mark.parametrize("R", [1, 4, 5, 8, 9, 16, 17, 32, 33, 64])
+def test_selection_widths(R):
+    """Frequency-weighted selection with 4, 8, 16 or 32 lanes per shot (R up to
+    32) and beyond, an odd batch; at 0.09 some shots have no candidate and
+    some several."""
+    from paper_2605_14170_gb300 import mbbp
+    H = named_code("bb72").HZ
+    e, _ = oracle.sample(SEED + 4, 0, 77, 72, 0.09, "bsc")
+    s = oracle.syndrome(H, e)
+    llr = channel_llr(72, 0.09).astype(np.float32)
+    B = mbbp.mbbp_build_bases(H, R, SEED)
+    got = _decode(B, s, llr, 15, 0.625)
+    ref = oracle.mbbp_decode(H, B.sets, s, llr, 15, 0.625, precision="f32")
+    assert 0 < ref["success"].sum()
+    _assert_exact(got, ref)
+
+
+@pytest.mark.parametrize("L", [6, 30, 48, 80, 81, 159, 160, 162])
+def test_syndrome_and_judge_mask_kernels(L):
+    """Syndromes and judge codes where the mask kernels' sizes end (160
+    variables and 96 rows; 320 and 160) and past them, against the
+    definitions."""
+    import torch
+    from paper_2605_14170_gb300 import mbbp
+    code = gb_code(L, [0, 1, 2], [0, 1, 2])  # k = 4 where 3 divides L
+    H, n = code.HZ, 2 * L
+    batch = 131
+    rng = np.random.default_rng(L)
+    e = (rng.random((batch, n)) < 0.1).astype(np.uint8)
+    ehat = e.copy()
+    ehat[::3] ^= (rng.random((len(ehat[::3]), n)) < 0.02).astype(np.uint8)  # mostly wrong syndromes
+    ops = mbbp.mbbp_logicals_build(H, code.HX)
+    lops = ops.ops()
+    flips = mbbp.mbbp_logicals_build(code.HX, H).ops()  # no syndrome, not stabilizers
+    assert ops.k == (4 if L % 3 == 0 else 0)
+    for i in range(1, batch, 3):  # a check of the other type, or also a logical operator
+        ehat[i] ^= code.HX[i % L]
+        if ops.k and i % 2:
+            ehat[i] ^= flips[i % ops.k]
+    sets = [[0]]
+    B = mbbp.mbbp_build_bases_from_sets(H, sets)
+    ep = torch.from_numpy(mbbp.pack_bits(e)).cuda()
+    s = torch.empty((batch, L), dtype=torch.uint8, device="cuda")
+    mbbp.mbbp_syndrome(B, ep, s)
+    assert np.array_equal(s.cpu().numpy(), (e.astype(int) @ H.T.astype(int) % 2).astype(np.uint8))
+    fail = torch.empty(batch, dtype=torch.uint8, device="cuda")
+    counts = torch.zeros(3, dtype=torch.int64, device="cuda")
+    mbbp.mbbp_judge(ops, ep, torch.from_numpy(ehat).cuda(), fail, counts)
+    r = (e ^ ehat).astype(int)
+    bad = (r @ H.T.astype(int) % 2).any(1)
+    odd = (r @ lops.T.astype(int) % 2).any(1) if ops.k else np.zeros(batch, bool)
+    want = np.where(bad, 1, np.where(odd, 2, 0))
+    assert bad.any() and not bad.all() and (not ops.k or (want == 2).any())
+    assert np.array_equal(fail.cpu().numpy(), want)
+    assert np.array_equal(counts.cpu().numpy(), np.bincount(want, minlength=3))
