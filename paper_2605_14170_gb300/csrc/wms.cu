@@ -155,7 +155,7 @@ __device__ __forceinline__ void wms_var_pass(const DevBases& B, int b, const uin
 // (pair of edge j of row r at float2 index row_slot(r) + 32 j: one coalesced
 // load per edge).  With G warps per item the thread with group index gt takes
 // rows gt, gt + 32 G, ...; bit k of sb is the syndrome bit of its k-th row.
-template <int DC, int G = 1, bool SLOT = false>
+template <int DC, int G = 1, bool SLOT = false, bool REG = false>
 __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const uint32_t* rinfo,
                                                int Mb, uint32_t sb, const float* q, float* m,
                                                const float* wt, const float* gt) {
@@ -166,12 +166,12 @@ __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const u
     for (int k = 0; k < (MP + GT - 1) / GT; ++k) {
         const int r = lane + GT * k;
         if (r >= Mb) continue;
-        const int deg = B.regular ? DC : (int)((__ldg(rinfo + r) >> 16) & 0xffu);
+        const int deg = (REG || B.regular) ? DC : (int)((__ldg(rinfo + r) >> 16) & 0xffu);
         const int e0 = SLOT ? 0 : __ldg(rp + r);
         const int rs = generic_bp::row_slot<DC>(r);
         float qq[DC];
 #pragma unroll
-        for (int j = 0; j < DC; ++j) qq[j] = (j < deg) ? q[rs + 32 * j] : MBBP_LMAX;
+        for (int j = 0; j < DC; ++j) qq[j] = (REG || j < deg) ? q[rs + 32 * j] : MBBP_LMAX;
         // the min over the other edges (and LMAX) with their sign product
         // (no q is -0: the LLRs enter as mu + 0), exact; the syndrome's sign
         // joins below
@@ -180,7 +180,7 @@ __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const u
         excluded_min<DC>(qq, x);
 #pragma unroll
         for (int j = 0; j < DC; ++j) {
-            if (j >= deg) continue;
+            if (!REG && j >= deg) continue;
             const float smn = __uint_as_float(__float_as_uint(x[j]) ^ sx);
             float wj, gg;
             if constexpr (SLOT) {
@@ -206,7 +206,7 @@ __device__ __forceinline__ void wms_check_pass(const DevBases& B, int b, const u
 // mu, and mu enters as llr + 0).  The arguments come by value (taken by
 // reference from the kernel's parameter, the decode on a length-882 code
 // measured 5% slower).
-template <int DC, int DV, int G, bool DEC>
+template <int DC, int DV, int G, bool DEC, bool REG>
 __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long group_item[kWmsWarps];
@@ -310,12 +310,12 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
             const int tp = min(it, a.T - 1);  // iterations past T reuse the last weights
             if (DEC) {
                 const float2* wgt = a.wg + ((size_t)b * a.T + tp) * DC * MP;
-                wms_check_pass<DC, G, true>(B, b, rinfo, Mb, sb, q, m, reinterpret_cast<const float*>(wgt),
+                wms_check_pass<DC, G, true, REG>(B, b, rinfo, Mb, sb, q, m, reinterpret_cast<const float*>(wgt),
                                             nullptr);
             } else {
                 const float* wt = a.w + ((size_t)b * a.T + tp) * a.E;
                 const float* gt = a.g + ((size_t)b * a.T + tp) * a.E;
-                wms_check_pass<DC, G>(B, b, rinfo, Mb, sb, q, m, wt, gt);
+                wms_check_pass<DC, G, false, REG>(B, b, rinfo, Mb, sb, q, m, wt, gt);
             }
             generic_bp::gsync<G>(bar);
             wms_var_pass<DV, G>(B, b, vd, m, q, mu, post);
@@ -365,22 +365,23 @@ __device__ __forceinline__ void wms_forward_items(const WmsArgs a) {
     }
 }
 
-// DEC: decode (halting rule, candidates), else the training forward.  Compiled
-// apart, since either one carried the other's tests and registers: decode on
-// [[288,12,18]] R = 8, 2,060 shots 548 -> 299 us, on the length-882 code R = 64,
-// 2,000 shots 7.16 -> 6.99 ms.  One warp per item: the compiler's own register
+// DEC: decode (halting rule, candidates), else the training forward; REG: every
+// row fills the kernel width.  Compiled apart, since each carried the others'
+// tests and registers: decode on [[288,12,18]] R = 8, 2,060 shots 548 -> 299
+// (DEC) -> 284 us (REG), on the length-882 code R = 64, 2,000 shots 7.16 -> 6.99
+// -> 6.83 ms.  One warp per item: the compiler's own register
 // choice.
-template <int DC, int DV, bool DEC>
+template <int DC, int DV, bool DEC, bool REG>
 __global__ void __launch_bounds__(kWmsWarps * 32) wms_forward_warp_kernel(const WmsArgs a) {
-    wms_forward_items<DC, DV, 1, DEC>(a);
+    wms_forward_items<DC, DV, 1, DEC, REG>(a);
 }
 
 // G > 1 warps per item: registers for three 8-warp blocks per SM, the
 // residency that the message areas allow for the codes that take G > 1
 // (without the bound the compiler stops at 64 registers and spills).
-template <int DC, int DV, int G, bool DEC>
+template <int DC, int DV, int G, bool DEC, bool REG>
 __global__ void __launch_bounds__(kWmsWarps * 32, 3) wms_forward_kernel(const WmsArgs a) {
-    wms_forward_items<DC, DV, G, DEC>(a);
+    wms_forward_items<DC, DV, G, DEC, REG>(a);
 }
 
 // SMEM_ST: the segment's recomputed states sit in shared memory after the
@@ -653,7 +654,7 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ gra
     p[i] = fminf(fmaxf(x, lo), hi);
 }
 
-template <int K, int G, bool DEC>
+template <int K, int G, bool DEC, bool REG>
 cudaError_t launch_forward_g(const WmsArgs& a, size_t fixed, size_t per_item, int warps, int per_sm,
                              cudaStream_t s, int sm_count) {
     const unsigned long long groups = (unsigned long long)(warps / G);
@@ -662,9 +663,9 @@ cudaError_t launch_forward_g(const WmsArgs& a, size_t fixed, size_t per_item, in
     unsigned long long grid = (unsigned long long)per_sm * sm_count;
     if (want < grid) grid = want;
     if constexpr (G == 1)
-        wms_forward_warp_kernel<K, K, DEC><<<(unsigned)grid, warps * 32, smem, s>>>(a);
+        wms_forward_warp_kernel<K, K, DEC, REG><<<(unsigned)grid, warps * 32, smem, s>>>(a);
     else
-        wms_forward_kernel<K, K, G, DEC><<<(unsigned)grid, warps * 32, smem, s>>>(a);
+        wms_forward_kernel<K, K, G, DEC, REG><<<(unsigned)grid, warps * 32, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -673,14 +674,14 @@ cudaError_t launch_forward_g(const WmsArgs& a, size_t fixed, size_t per_item, in
 // KB of shared memory per block (for the decode H's columns once, then one area
 // per item); a larger G only when it holds at least half again as many warps
 // as the best smaller one
-template <int K, bool DEC>
+template <int K, bool DEC, bool REG>
 cudaError_t launch_forward(const WmsArgs& a, cudaStream_t s, int sm_count) {
     const WmsLayout L = wms_layout(K, a.B.MP, a.B.n, a.ckpt);
     if (L.fwd_bytes > 200 * 1024) return cudaErrorInvalidConfiguration;
     const size_t fixed = (size_t)((K * a.B.mpad * 2 + 15) & ~15);
-    const void* kerns[3] = {reinterpret_cast<const void*>(wms_forward_warp_kernel<K, K, DEC>),
-                            reinterpret_cast<const void*>(wms_forward_kernel<K, K, 2, DEC>),
-                            reinterpret_cast<const void*>(wms_forward_kernel<K, K, 4, DEC>)};
+    const void* kerns[3] = {reinterpret_cast<const void*>(wms_forward_warp_kernel<K, K, DEC, REG>),
+                            reinterpret_cast<const void*>(wms_forward_kernel<K, K, 2, DEC, REG>),
+                            reinterpret_cast<const void*>(wms_forward_kernel<K, K, 4, DEC, REG>)};
     int best_g = -1, best_w = 0, best_b = 0;
     for (int gi = 0; gi < 3; ++gi) {
         const int G = 1 << gi;
@@ -701,14 +702,16 @@ cudaError_t launch_forward(const WmsArgs& a, cudaStream_t s, int sm_count) {
         }
     }
     if (best_g < 0) return cudaErrorInvalidConfiguration;
-    if (best_g == 0) return launch_forward_g<K, 1, DEC>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
-    if (best_g == 1) return launch_forward_g<K, 2, DEC>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
-    return launch_forward_g<K, 4, DEC>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
+    if (best_g == 0) return launch_forward_g<K, 1, DEC, REG>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
+    if (best_g == 1) return launch_forward_g<K, 2, DEC, REG>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
+    return launch_forward_g<K, 4, DEC, REG>(a, fixed, L.fwd_bytes, best_w, best_b, s, sm_count);
 }
 
 template <int K>
 cudaError_t launch_wms_t(const WmsArgs& a, bool backward, cudaStream_t s, int sm_count) {
-    if (!backward) return a.decode ? launch_forward<K, true>(a, s, sm_count) : launch_forward<K, false>(a, s, sm_count);
+    if (!backward && a.decode)
+        return a.B.regular ? launch_forward<K, true, true>(a, s, sm_count) : launch_forward<K, true, false>(a, s, sm_count);
+    if (!backward) return launch_forward<K, false, false>(a, s, sm_count);
     const WmsLayout L = wms_layout(K, a.B.MP, a.B.n, a.ckpt);
     const size_t st_bytes = (size_t)a.ckpt * L.S * 4;
     const bool smem_st = wms_states_in_smem(a.B, a.ckpt);
