@@ -409,10 +409,9 @@ BankLayout bank_layout(const Tanner& g, const std::vector<int>& src, int n, int 
 
 // Row positions for the serial chunk kernel.  In a layer the kernel spreads
 // (row, shot) pairs over the lanes, 32 / CS rows per lane step; for edge j of
-// its row a lane stores to slot j * MP + pos(row) and gathers the messages of
-// the edge's variable from the slots j' * MP + pos(row') of its other rows.
-// With MP a multiple of 32, slot s of shot sh sits in bank
-// (pos + 4 sh) mod 32, so the accesses of one instruction conflict when the
+// its row a lane stores to the slot of (pos(row), j) and gathers the messages of
+// the edge's variable from those of (pos(row'), j') of its other rows.  A slot of
+// position pos of shot sh sits in bank (pos + 4 sh) mod 32, so the accesses of one instruction conflict when the
 // positions they touch collide mod 32.  Simulated annealing over a
 // permutation of the positions 0..M-1 minimizes the summed worst bank load
 // of every (layer, lane step, j, access) group; the arithmetic is unchanged

@@ -17,14 +17,16 @@ constexpr size_t kStaticScratchBytes = MBBP_NOALLOC_SCRATCH_BYTES;
 inline int words_for(int n) { return (n + 31) / 32; }
 inline int round_up(int x, int a) { return (x + a - 1) / a * a; }
 
-// Device copy of the R representations of one code.  Rows of H^(t) are laid
-// out ELL-style: the j-th edge of row r of representation t is "slot"
-// j * MP + r of that representation's message array, so lane r of a warp
-// reads the j-th message of its row with unit stride across the warp.
+// Device copy of the R representations of one code.  The rows of H^(t) are at
+// positions (a permutation within each block of 32 rows, chosen by the host to
+// spread the variable pass over the shared-memory banks); edge j of the row at
+// position r is message slot (r / 32) * 32 DC + 32 j + r % 32, so lane r % 32 of
+// a warp reads the edges of its row with unit stride across the warp, at
+// constant offsets from one address.  Tables "by row" below are by position.
 struct DevBases {
     const uint32_t* rowinfo;  // [R][MP] src row (bits 0-15) | degree (16-23) | valid (bit 31)
     const uint2* vdesc;       // [R][n]  x = first slot-list entry, y = variable | degree << 16;
-                              //         variables sorted by degree (stable)
+                              //         variables by ascending degree, placed like the rows
     const uint16_t* vslot;    // slot ids of every variable, ascending row of H^(t)
     const uint4* vdesc6;      // width 6 only: [R][n] in vdesc order, x = vdesc.y, y/z/w = byte
                               //         offsets (4 * slot id) of the variable's slots, 2 per word
