@@ -431,6 +431,8 @@ cudaError_t prepare_kernel(const void* func, int threads, size_t smem, int* bloc
 
 cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     if (a.B.shape != 0) return launch_decode_small(a, s, sm_count);
+    const cudaError_t e = cudaMemsetAsync(a.counter, 0, sizeof(unsigned long long), s);
+    if (e != cudaSuccess) return e;
     const int K = a.B.DC;
     if (a.rule == MBBP_RULE_NMS) {
         if (K == 6) return launch_decode_k<6, MBBP_RULE_NMS>(a, s, sm_count);

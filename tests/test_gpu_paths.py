@@ -128,6 +128,35 @@ def test_small_code_run_lengths(shots):
     _assert_exact(got, oracle.mbbp_decode(H, B.sets, s, llr, 25, 0.625, precision="f32"))
 
 
+@pytest.mark.parametrize("code", ["bb72", "bb144"])
+def test_small_code_item_per_warp(code):
+    """The small-code kernel without work pulls, up to and beyond the most
+    items that the resident warps hold at one each (152 SMs x 20 to 24 warps,
+    R = 64: 47 to 57 shots); the workspace holds ones, as a call finds it."""
+    import torch
+    from paper_2605_14170_gb300 import mbbp
+    H = named_code(code).HZ
+    n = H.shape[1]
+    e, _ = oracle.sample(SEED + 8, 0, 64, n, 0.05, "bsc")
+    s = oracle.syndrome(H, e)
+    llr = channel_llr(n, 0.05).astype(np.float32)
+    B = mbbp.mbbp_build_bases(H, 64, SEED)
+    ref = oracle.mbbp_decode(H, B.sets, s, llr, 25, 0.625, precision="f32")
+    for shots in (1, 40, *range(45, 60), 64):
+        ws = torch.full((mbbp.mbbp_decode_workspace_size(B, shots),), 255, dtype=torch.uint8, device="cuda")
+        got = {"e_hat": torch.zeros((shots, n), dtype=torch.uint8), "conv": torch.zeros((shots, 64), dtype=torch.uint8),
+               "success": torch.zeros(shots, dtype=torch.uint8), "selected": torch.zeros(shots, dtype=torch.int16),
+               "iters": torch.zeros((shots, 64), dtype=torch.int16)}
+        got = {k: v.cuda() for k, v in got.items()}
+        mbbp.mbbp_decode(B, torch.from_numpy(s[:shots]).cuda(), torch.from_numpy(llr).cuda(), 25, 0.625,
+                         mbbp.RULE_NMS, got["e_hat"], got["conv"], got["success"], ws, iters_run=got["iters"],
+                         selected=got["selected"])
+        torch.cuda.synchronize()
+        for key, rkey in (("e_hat", "ehat"), ("conv", "conv"), ("success", "success"), ("selected", "selected"),
+                          ("iters", "iters")):
+            assert np.array_equal(got[key].cpu().numpy(), ref[rkey][:shots]), (key, shots)
+
+
 @pytest.mark.parametrize("rule", ["nms", "sp"])
 @pytest.mark.parametrize("code,R,shots", [("bb72", 64, 2000), ("irregular", 64, 2003), ("gb90w4", 20, 1001),
                                           ("gb166", 8, 1300)])
