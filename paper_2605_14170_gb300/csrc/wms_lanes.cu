@@ -40,7 +40,7 @@ constexpr int kLaneShots = 32 / kLaneRows;
 struct LanesLayout {
     int rsteps, npos;                      // row steps, variable positions
     int vt, e0, sw, et, part, a0, a1, gp;  // tables, two message arrays, the posterior gradients
-    int slot_floats, total;
+    int slot_floats, total;                // floats of a message array: the slots, then 32 that are only read
 };
 
 // Words of a variable's record: mu, the variable, DC offsets.
@@ -57,7 +57,7 @@ __host__ __device__ inline LanesLayout lanes_layout(int DC, int MP, int n) {
     L.et = L.sw + L.rsteps * 4;
     L.part = L.et + L.npos / S * 4;
     L.a0 = (L.part + kLaneThreads * 4 + 127) & ~127;
-    L.slot_floats = L.rsteps * DC * 32;
+    L.slot_floats = L.rsteps * DC * 32 + 32;
     L.a1 = L.a0 + L.slot_floats * 4;
     L.gp = L.a1 + L.slot_floats * 4;
     L.total = L.gp + L.npos / S * 128;
@@ -176,12 +176,17 @@ struct Block {
             int np = pos[deg] + idx;
             const int last = (idx == cnt[deg] - 1) ? pos[deg + 1] : np + 1;
             // a class is padded to whole warp steps with copies of its last
-            // variable (same loads, same stores; bit 31 keeps it out of sums)
+            // variable, marked by bit 31.  They store nothing and read the row
+            // behind the slots, which nobody writes: the two halves of a warp
+            // on one variable would read and write its words unordered (the
+            // adjoint's gradient could be added twice).  Predicated stores,
+            // since a branch around the copies took the step on [[144,12,12]],
+            // batch 4096, from 2.72 to 2.82 ms.
             for (uint32_t dup = 0; np < last; ++np, dup = 0x80000000u) {
                 uint32_t* rec = vt() + np * RW;
                 for (int i = 0; i < DC; ++i) {
-                    uint32_t off = 0;
-                    if (i < deg) {
+                    uint32_t off = (uint32_t)(L.rsteps * (DC * 128));
+                    if (i < deg && !dup) {
                         const int s = __ldg(B.vslot + d.x + i);
                         const int r = (s / (32 * DC)) * 32 + (s & 31), j = (s >> 5) % DC;
                         off = (uint32_t)((r / S) * (DC * 128) + j * 128 + (r % S) * (4 * CS));
@@ -267,10 +272,11 @@ struct Block {
         }
     }
 
-    // q^(t) of one variable of degree D from its messages m (arr0 at off).
+    // q^(t) of one variable of degree D from its messages m (arr0 at off);
+    // own: not a padding copy.
     template <int D>
     __device__ __forceinline__ float var_q(const uint32_t (&off)[D > 0 ? D : 1], const float (&m)[D > 0 ? D : 1],
-                                           float mu) const {
+                                           float mu, bool own) const {
         char* q0 = arr0() + 4 * slot;
         float P = mu;
 #pragma unroll
@@ -278,7 +284,7 @@ struct Block {
             float q = P;
 #pragma unroll
             for (int k = i + 1; k < D; ++k) q = __fadd_rn(q, m[k]);
-            *reinterpret_cast<float*>(q0 + off[i]) = q;
+            if (own) *reinterpret_cast<float*>(q0 + off[i]) = q;
             P = __fadd_rn(P, m[i]);
         }
         return P;
@@ -324,10 +330,11 @@ __global__ void __launch_bounds__(kLaneThreads, 1) wms_forward_lanes_kernel(cons
         if (b != k.b) k.load_rep(b, cls);
         k.load_shots(blk, batch);
         // q^(0) = mu, m^(0) = 0
-        k.var_pass([&]<int D>(int, const uint32_t(&off)[D > 0 ? D : 1], float mu, uint32_t) {
+        k.var_pass([&]<int D>(int, const uint32_t(&off)[D > 0 ? D : 1], float mu, uint32_t v) {
             char* q0 = k.arr0() + 4 * k.slot;
 #pragma unroll
-            for (int i = 0; i < D; ++i) *reinterpret_cast<float*>(q0 + off[i]) = mu;
+            for (int i = 0; i < D; ++i)
+                if (!(v >> 31)) *reinterpret_cast<float*>(q0 + off[i]) = mu;
         });
         for (int i = threadIdx.x; i < k.rsteps * (DC * 32); i += blockDim.x) reinterpret_cast<float*>(M)[i] = 0.0f;
         __syncthreads();
@@ -348,13 +355,12 @@ __global__ void __launch_bounds__(kLaneThreads, 1) wms_forward_lanes_kernel(cons
                 float m[D > 0 ? D : 1];
 #pragma unroll
                 for (int i = 0; i < D; ++i) m[i] = *reinterpret_cast<const float*>(m0 + off[i]);
-                const float post = k.template var_q<D>(off, m, mu);
+                const float post = k.template var_q<D>(off, m, mu, !(v >> 31));
                 if (bce) {
                     const float x = bce_neg_sigmoid(post, (int)((k.et()[st] >> k.lane) & 1u));
                     if (!(v >> 31)) lacc += x;
                 }
-                if (last && a.post && k.live)
-                    a.post[((size_t)k.shot * B.R + b) * B.n + (v & 0xffffu)] = post;
+                if (last && a.post && k.live && !(v >> 31)) a.post[((size_t)k.shot * B.R + b) * B.n + v] = post;
             });
             __syncthreads();
         }
@@ -414,7 +420,8 @@ __global__ void __launch_bounds__(kLaneThreads, 1) wms_backward_lanes_kernel(con
             const float sig = 1.0f / (1.0f + expf(pv));
             const float gp = lwl * ((float)((k.et()[st] >> k.lane) & 1u) - sig);
 #pragma unroll
-            for (int i = 0; i < D; ++i) *reinterpret_cast<float*>(g0 + off[i]) = gp;
+            for (int i = 0; i < D; ++i)
+                if (!(v >> 31)) *reinterpret_cast<float*>(g0 + off[i]) = gp;
         });
         const int nseg = (a.T + a.ckpt - 1) / a.ckpt;
         for (int sg = nseg - 1; sg >= 0; --sg) {
@@ -432,12 +439,12 @@ __global__ void __launch_bounds__(kLaneThreads, 1) wms_backward_lanes_kernel(con
             __syncthreads();
             for (int t = t0 + 1; t < t1; ++t) {
                 const char* mp = state(t - 1 - t0);
-                k.var_pass([&]<int D>(int, const uint32_t(&off)[D > 0 ? D : 1], float mu, uint32_t) {
+                k.var_pass([&]<int D>(int, const uint32_t(&off)[D > 0 ? D : 1], float mu, uint32_t v) {
                     const char* m0 = mp + 4 * k.slot;
                     float m[D > 0 ? D : 1];
 #pragma unroll
                     for (int i = 0; i < D; ++i) m[i] = *reinterpret_cast<const float*>(m0 + off[i]);
-                    k.template var_q<D>(off, m, mu);
+                    k.template var_q<D>(off, m, mu, !(v >> 31));
                 });
                 __syncthreads();
                 const float* wt = a.w + ((size_t)b * a.T + (t - 1)) * a.E;
@@ -450,7 +457,7 @@ __global__ void __launch_bounds__(kLaneThreads, 1) wms_backward_lanes_kernel(con
             // first the adjoint of the variable pass of iteration t + 1's q,
             // which the same thread owns
             auto var_both = [&](const char* mp, bool adjoint, bool forward) {
-                k.var_pass([&]<int D>(int st, const uint32_t(&off)[D > 0 ? D : 1], float mu, uint32_t) {
+                k.var_pass([&]<int D>(int st, const uint32_t(&off)[D > 0 ? D : 1], float mu, uint32_t v) {
                     constexpr int DD = D > 0 ? D : 1;
                     const char* q0 = k.arr0() + 4 * k.slot;
                     char* g0 = GM + 4 * k.slot;
@@ -471,11 +478,12 @@ __global__ void __launch_bounds__(kLaneThreads, 1) wms_backward_lanes_kernel(con
 #pragma unroll
                         for (int i = 0; i < D; ++i) {
                             float* gm = reinterpret_cast<float*>(g0 + off[i]);
-                            *gm += G - gq[i] + gp;
+                            const float x = *gm + (G - gq[i] + gp);
+                            if (!(v >> 31)) *gm = x;
                         }
                     }
                     if (forward) {
-                        const float post = k.template var_q<D>(off, m, mu);
+                        const float post = k.template var_q<D>(off, m, mu, !(v >> 31));
                         if (a.all_iters)
                             GP[32 * st] =
                                 lwl * ((float)((k.et()[st] >> k.lane) & 1u) - 1.0f / (1.0f + expf(post)));
@@ -590,7 +598,7 @@ bool wms_lanes_fit(const DevBases& B, int batch) {
     // memory (the length-882 code's do not).
     const long long blocks = ((long long)batch + kLaneShots - 1) / kLaneShots;
     return (long long)batch * B.R >= 256 && blocks * B.R <= INT_MAX / 2 &&
-           lanes_layout(B.DC, B.MP, B.n).total <= 226 * 1024;
+           lanes_layout(B.DC, B.MP, B.n).total <= 226 * 1024 + 256;  // and 256 static
 }
 
 size_t wms_lanes_grid(const DevBases& B, int batch, int sm_count) {

@@ -113,6 +113,48 @@ def test_wms_training_one_shot_per_lane(code, ckpt, all_iters):
         assert np.linalg.norm(a - b) <= 1e-4 * np.linalg.norm(b)
 
 
+@pytest.mark.parametrize("ckpt,all_iters", [(1, False), (3, True), (6, True)])
+@pytest.mark.parametrize("code", ["bb72", "gb90w4", "irregular"])
+def test_wms_training_odd_variable_classes(code, ckpt, all_iters):
+    """87 shots at R = 3 (the kernels with one shot per lane), representations
+    with an odd number of variables of some degree: the step that such a
+    class fills by half adds to no variable twice.  Gradients against the
+    FP64 oracle's adjoint by norm: 1e-3 bounds FP32 rounding and the odd
+    near-tie of two minima, a variable counted twice moves the norm by one
+    part in sqrt(n) at least (5e-2 here)."""
+    import torch
+    from paper_2605_14170_gb300 import mbbp
+    H = named_code("bb72").HZ if code == "bb72" else CODES[code]()
+    n, T, batch, R, scale = H.shape[1], 6, 87, 3, 1e-3
+    e, _ = oracle.sample(SEED + 5, 0, batch, n, 0.05, "bsc")
+    s = oracle.syndrome(H, e)
+    B = mbbp.mbbp_build_bases(H, R, SEED)
+    degrees = [H.sum(0, dtype=int) + H[rows].sum(0, dtype=int) for rows in B.sets]
+    assert any((np.bincount(d) % 2).any() for d in degrees)
+    rng = np.random.default_rng(4)
+    E = int(B.edges.max())
+    w, g = (rng.uniform(lo, hi, (R, T, E)).astype(np.float32) for lo, hi in ((0.4, 1.0), (0.0, 0.4)))
+    mu = rng.uniform(1.5, 3.5, n).astype(np.float32)
+    ref = [np.zeros((R, T, E)) for _ in range(2)]
+    for shot in range(batch):
+        for b, rows in enumerate(B.sets):
+            Eb = int(B.edges[b])
+            grads = oracle.wms_backward(np.concatenate([H, H[rows]]), np.concatenate([s[shot], s[shot][rows]]), mu,
+                                        w[b][:, :Eb], g[b][:, :Eb], e[shot], scale, all_iters=all_iters)[1:]
+            for r, x in zip(ref, grads):
+                r[b][:, :Eb] += x
+    wt, gt, st, mt, et = (torch.from_numpy(x).cuda() for x in (w, g, s, mu, mbbp.pack_bits(e)))
+    post = torch.empty((batch, R, n), device="cuda")
+    gw, gg = torch.zeros_like(wt), torch.zeros_like(gt)
+    ws = torch.empty(mbbp.mbbp_wms_workspace_size(B, batch, T, ckpt), dtype=torch.uint8, device="cuda")
+    mbbp.mbbp_wms_forward(B, st, mt, T, wt, gt, ckpt, et, scale, post, None, ws, all_iters=all_iters)
+    mbbp.mbbp_wms_backward(B, st, mt, T, wt, gt, ckpt, et, scale, post, gw, gg, ws, all_iters=all_iters)
+    torch.cuda.synchronize()
+    for got, r in zip((gw, gg), ref):
+        assert np.linalg.norm(r) > 0
+        assert np.linalg.norm(got.double().cpu().numpy() - r) <= 1e-3 * np.linalg.norm(r)
+
+
 @pytest.mark.parametrize("shots", [1, 3, 200, 1601])
 def test_small_code_run_lengths(shots):
     """The small-code kernel's runs of 8, 2 and 1 shots ([[72]], R = 64: the
