@@ -35,6 +35,15 @@ constexpr uint32_t kSlots = (1u << kShots) - 1u;
 constexpr int kRing = 32;            // tickets (shot numbers) a group holds, at most
 constexpr int kPool = kShots;        // tickets kept ahead of need
 
+// Shared memory of fixed size; with the layout below it may fill what a block
+// can have.
+struct SerialLanesFixed {
+    int cls_cnt[16], cls_first[16], cls_pos[16];
+    int open;
+    uint32_t unsat[kGroups][2];
+};
+constexpr int kMaxDynamic = 227 * 1024 - (((int)sizeof(SerialLanesFixed) + 127) & ~127);
+
 // Byte offsets in shared memory.
 struct SerialLanesLayout {
     int rec, var, cnt, src, hidx, hpos, posof, lptr, group0;  // tables of the block
@@ -119,9 +128,8 @@ __device__ __forceinline__ void lane_posts(int& st, int nw, const int* cend, con
 template <int DC, int RULE, bool REG>
 __global__ void __launch_bounds__(kMaxThreads, 1) decode_serial_lanes_kernel(const DecodeArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ int cls_cnt[16], cls_first[16], cls_pos[16];
-    __shared__ int s_open;
-    __shared__ uint32_t s_unsat[kGroups][2];
+    __shared__ SerialLanesFixed fixed;
+    int *cls_cnt = fixed.cls_cnt, *cls_first = fixed.cls_first, *cls_pos = fixed.cls_pos;
     const DevBases& B = a.B;
     const ShotIO& io = a.io;
     const int n = B.n, m = B.m, R = B.R, W = B.W, MP = B.MP;
@@ -145,7 +153,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1) decode_serial_lanes_kernel(con
     uint32_t* ew = reinterpret_cast<uint32_t*>(area + L.ew);
     uint32_t* sw = reinterpret_cast<uint32_t*>(area + L.sw);
     int* ring = reinterpret_cast<int*>(area + L.ring);
-    uint32_t* unsat = s_unsat[grp];
+    uint32_t* unsat = fixed.unsat[grp];
     // blocks start spread over the representations by their rows
     if (threadIdx.x == 0) {
         long long total = 0, sum = 0;
@@ -153,21 +161,21 @@ __global__ void __launch_bounds__(kMaxThreads, 1) decode_serial_lanes_kernel(con
         const long long at = total * (2 * (long long)blockIdx.x + 1) / (2 * (long long)gridDim.x);
         int t = 0;
         while (t + 1 < R && (sum += __ldg(B.rows + t)) <= at) ++t;
-        s_open = t;
+        fixed.open = t;
     }
     __syncthreads();
-    const int b0 = s_open;
+    const int b0 = fixed.open;
 
     for (int kb = 0; kb < R; ++kb) {
         __syncthreads();
         const int b = (b0 + kb) % R;
         if (threadIdx.x == 0) {
-            s_open = *reinterpret_cast<volatile unsigned int*>(a.rep_counter + b) < (unsigned)io.batch;
+            fixed.open = *reinterpret_cast<volatile unsigned int*>(a.rep_counter + b) < (unsigned)io.batch;
         }
         if (threadIdx.x < 16) cls_cnt[threadIdx.x] = 0;
         if (gt < 2) unsat[gt] = 0;
         __syncthreads();
-        if (!s_open) continue;
+        if (!fixed.open) continue;
         // tables of representation b; rows in layer order, layers padded to
         // whole steps.  Until the shots start, the first group's message area
         // holds the row of each position of the chunk layout and, per row, the
@@ -515,7 +523,7 @@ cudaError_t launch_decode_serial_lanes(const DecodeArgs& a, cudaStream_t s, int 
     const DevBases& B = a.B;
     *taken = false;
     if (a.io.post || a.io.llr_stride != 0 || !B.edesc) return cudaSuccess;
-    if (serial_lanes_layout(B.DC, B.lsteps, B.m, B.n).total > 227 * 1024) return cudaSuccess;
+    if (serial_lanes_layout(B.DC, B.lsteps, B.m, B.n).total > kMaxDynamic) return cudaSuccess;
     if (B.DC == 6) return launch_width<6>(a, s, sm_count, taken);
     if (B.DC == 8) return launch_width<8>(a, s, sm_count, taken);
     return cudaSuccess;

@@ -228,6 +228,40 @@ def test_serial_one_shot_per_lane(code, R, shots, rule):
                                               schedule=oracle.SCHEDULE_SERIAL))
 
 
+SERIAL_LIMIT = {
+    # code, rows of H repeated in every representation: bytes of shared memory
+    # that the one-shot-per-lane layout takes besides 256 of fixed size, of
+    # 232448 in all
+    "230528": (lambda: gb_code(160, [0, 7, 31], [2, 19, 55]).HZ, lambda H: [list(range(53))] * 64),
+    "232320": (lambda: gb_code(144, [76, 90, 106, 132], [56, 104, 112, 138]).HZ,
+               lambda H: oracle.collect_subtrees(H, 20, 20260514)),
+    "232448": (lambda: gb_code(160, [0, 7, 31], [2, 19, 55]).HZ, lambda H: [list(range(54))] * 64),
+}
+
+
+@pytest.mark.parametrize("size", sorted(SERIAL_LIMIT))
+def test_serial_one_shot_per_lane_shared_memory_limit(size):
+    """Serial batches of codes on both sides of the shared memory that the
+    one-shot-per-lane kernel may take: decoded, bit for bit as by the
+    warp-per-slot kernel (which the same LLRs given per shot take) and, for
+    the first shots, by the FP32 oracle."""
+    from paper_2605_14170_gb300 import mbbp
+    code, rows = SERIAL_LIMIT[size]
+    H = code()
+    n, sets = H.shape[1], rows(H)
+    shots = 84_000 // len(sets)
+    e, _ = oracle.sample(SEED + 6, 0, shots, n, 0.08, "bsc")
+    s = oracle.syndrome(H, e)
+    llr = channel_llr(n, 0.08).astype(np.float32)
+    B = mbbp.mbbp_build_bases_from_sets(H, sets)
+    got = _decode(B, s, llr, 8, 0.8, schedule=mbbp.SCHEDULE_SERIAL)
+    ref = _decode(B, s, np.tile(llr, (shots, 1)), 8, 0.8, schedule=mbbp.SCHEDULE_SERIAL)
+    for key in ("conv", "iters", "cand", "selected", "success", "e_hat"):
+        assert np.array_equal(got[key], ref[key]), key
+    few = oracle.mbbp_decode(H, sets, s[:16], llr, 8, 0.8, precision="f32", schedule=oracle.SCHEDULE_SERIAL)
+    _assert_exact({k: v[:16] for k, v in got.items()}, few)
+
+
 @pytest.mark.parametrize("R", [1, 4, 5, 8, 9, 16, 17, 32, 33, 64])
 def test_selection_widths(R):
     """Frequency-weighted selection with 4, 8, 16 or 32 lanes per shot (R up to
