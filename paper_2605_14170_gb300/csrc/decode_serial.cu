@@ -1,6 +1,7 @@
-// Serial-schedule launches (Section II-B).  Batches long enough for it take
-// the one-shot-per-lane kernel (decode_serial_lanes.cu); per-shot LLRs, calls
-// for posteriors, short batches and long codes stay here.  Widths 6 and 8 use the
+// Serial-schedule launches (Section II-B).  Long batches of shots that are not
+// easy take the one-shot-per-lane kernel (decode_serial_lanes.cu has the rule);
+// per-shot LLRs, calls for posteriors, short or easy batches and long codes
+// stay here.  Widths 6 and 8 use the
 // slot path of bp_serial.cuh: a persistent grid whose warps pull shots of
 // one representation at a time from per-representation counters and decode
 // CS of them at once (CS = 4, 2 or 1, the largest that leaves about half of
@@ -19,6 +20,7 @@ constexpr int kSerialMinBlocks = 3;
 template <int DC, int NO, int NV, int RULE, bool REG, int CS>
 __global__ void __launch_bounds__(kSerialWarps * 32, kSerialMinBlocks)
 decode_serial_chunk_kernel(const DecodeArgs a) {
+    if (a.lanes && *a.lanes) return;  // the one-shot-per-lane kernel takes the call
     extern __shared__ __align__(16) unsigned char smem[];
     const DevBases& B = a.B;
     const int warp = warp_index();
@@ -84,11 +86,14 @@ cudaError_t launch_width(const DecodeArgs& a, cudaStream_t s, int sm_count) {
 
 }  // namespace
 
-cudaError_t launch_decode_serial(const DecodeArgs& a, cudaStream_t s, int sm_count) {
-    if (!a.B.edesc || (a.B.DC != 6 && a.B.DC != 8)) return launch_decode_serial_generic(a, s, sm_count);
-    bool taken = false;
-    const cudaError_t e = launch_decode_serial_lanes(a, s, sm_count, &taken);
-    if (e != cudaSuccess || taken) return e;
+cudaError_t launch_decode_serial(const DecodeArgs& args, cudaStream_t s, int sm_count) {
+    if (!args.B.edesc || (args.B.DC != 6 && args.B.DC != 8)) {
+        const cudaError_t e = cudaMemsetAsync(args.counter, 0, sizeof(unsigned long long), s);
+        return e == cudaSuccess ? launch_decode_serial_generic(args, s, sm_count) : e;
+    }
+    DecodeArgs a = args;
+    const cudaError_t e = launch_decode_serial_lanes(args, s, sm_count, &a.lanes);
+    if (e != cudaSuccess) return e;
     const bool reg = a.B.regular != 0;
     if (a.rule == MBBP_RULE_NMS)
         return reg ? launch_width<MBBP_RULE_NMS, true>(a, s, sm_count)

@@ -1,4 +1,5 @@
-// Serial schedule (Section II-B), one shot per lane, kernel widths 6 and 8: a
+// Serial schedule (Section II-B), one shot per lane, kernel widths 6 and 8, for
+// long batches of shots that are not easy (the rule is at serial_route_kernel): a
 // block decodes the shots of one representation in two groups of warps, each
 // 16 shots in lockstep, two rows of a layer per warp step.  A slot whose shot
 // halts takes the next one from the representation's counter, so lanes do not
@@ -20,6 +21,7 @@
 // Serial + least metric, p = 0.06, R = 20: [[288,12,18]], 20,000 shots 23.65 ->
 // 13.9 ms; [[144,12,12]], 40,000 shots 17.4 -> 8.7 ms.
 #include <algorithm>
+#include <cmath>
 
 #include "bp_generic.cuh"
 
@@ -125,8 +127,62 @@ __device__ __forceinline__ void lane_posts(int& st, int nw, const int* cend, con
     if constexpr (D < DC) lane_posts<D + 1, DC>(st, nw, cend, ms, var, ew);
 }
 
+// Which of the two serial kernels takes a call.  A shot that halts here makes
+// its block refill a slot and the last shots of a representation run at this
+// kernel's pace per iteration, 2-3 times slower than a warp per slot; both are
+// small beside the iterations of a long batch whose shots take several.  How
+// many they take shows in the syndromes, which are on the device: so one block
+// counts the ones of 128 of them, spread over the batch, sets *flag, and of the
+// two kernels launched after it the other returns at once.  It also clears the
+// counters, so a call pays for one empty launch more (AAA).
+//
+// min-sum: rounds * density^2 >= 1 and density >= 0.1, a round being 32 items
+// (one block's slots) per SM.  Measured against the warp-per-slot kernel
+// (13 codes of length 60 to 288, rows of weight 2 to 8, R = 4 to 20, error
+// rates 0.001 to 0.2, alpha 0.625 and 0.875, 1 to 100 iterations): no point
+// that satisfies the rule is slower.  Worst and best of the codes with rows of
+// weight 6, 100 iterations, by density (0.056: 1%, 0.11: 2%, 0.20: 4%, 0.27: 6%,
+// 0.32: 8% errors) and rounds:
+//              4          16         32         96
+//   0.056      -       0.68-1.12  0.85-1.1  0.86-1.16
+//   0.11       -       0.73-1.12  0.84-1.29  1.04-1.83
+//   0.20       -       0.90-1.82  1.03-2.08  1.18-2.51
+//   0.27   0.77-1.33   1.06-2.19  1.21-2.56  -
+//   0.32   0.88-1.52   1.22-2.59  1.28-2.85  -
+// Sum-product shots take longer in one lane: rounds * density^2 >= 4 and
+// density >= 0.2 (0.2, 64 rounds: 0.97-2.0; 0.32, 16 rounds: 0.91-2.2, 64:
+// 1.10-2.4).
+constexpr int kRouteShots = 128;
+constexpr int kRouteThreads = 1024;
+constexpr int kMinRounds = 16;
+
+float min_density(int rule, double rounds) {
+    return rule == MBBP_RULE_NMS ? std::max(0.1f, (float)std::sqrt(1.0 / rounds))
+                                 : std::max(0.2f, (float)std::sqrt(6.0 / rounds));
+}
+
+__global__ void __launch_bounds__(kRouteThreads) serial_route_kernel(const uint8_t* __restrict__ synd, int m, int batch,
+                                                                     int R, float density, unsigned int* flag,
+                                                                     unsigned int* rep_counter) {
+    __shared__ int ones;
+    if (threadIdx.x == 0) ones = 0;
+    if (threadIdx.x < R) rep_counter[threadIdx.x] = 0;
+    __syncthreads();
+    const int shots = min(batch, kRouteShots), step = batch / shots;
+    int c = 0;
+    for (int i = threadIdx.x; i < shots * m; i += kRouteThreads) {
+        const int k = i / m;
+        c += __ldg(synd + (size_t)(k * step) * m + (i - k * m)) & 1;
+    }
+    c = __reduce_add_sync(kFull, c);
+    if ((threadIdx.x & 31) == 0) atomicAdd(&ones, c);
+    __syncthreads();
+    if (threadIdx.x == 0) *flag = (float)ones >= density * (float)(shots * m);
+}
+
 template <int DC, int RULE, bool REG>
 __global__ void __launch_bounds__(kMaxThreads, 1) decode_serial_lanes_kernel(const DecodeArgs a) {
+    if (!*a.lanes) return;
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ SerialLanesFixed fixed;
     int *cls_cnt = fixed.cls_cnt, *cls_first = fixed.cls_first, *cls_pos = fixed.cls_pos;
@@ -476,57 +532,55 @@ __global__ void __launch_bounds__(kMaxThreads, 1) decode_serial_lanes_kernel(con
     }
 }
 
-// Launches the call, unless the batch is too short for it (*taken = false).
+// Launches the kernel with 24 warps per SM in as many blocks as an SM holds, 1
+// to 4: more blocks hide each other's barriers and hold more shots ([[72]] R = 20
+// at p = 0.06, 48 rounds, against the warp-per-slot kernel: 1 / 2 / 3 / 4 blocks
+// 0.84 / 1.20 / 1.32 / 1.33 times as fast).
 template <int DC, int RULE, bool REG>
-cudaError_t launch_t(const DecodeArgs& a, cudaStream_t s, int sm_count, bool* taken) {
+cudaError_t launch_t(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     auto kern = decode_serial_lanes_kernel<DC, RULE, REG>;
     const SerialLanesLayout L = serial_lanes_layout(DC, a.B.lsteps, a.B.m, a.B.n);
-    // 24 warps per SM: as many blocks as shared memory holds, 1 to 4.  A block
-    // holds 32 shots whatever its size, and the last shots of a representation
-    // run alone, so many blocks need many items: against the warp-per-slot
-    // kernel, [[72]] R = 8 at p = 0.04 and 0.015, 100,000 shots (41 rounds of
-    // the slots of 4 blocks per SM): 1.40x and 1.10x as fast (2 blocks: 1.18x and
-    // 0.93x), 20,000 shots at p = 0.015 (8 rounds) 0.99x (0.96x), 2,500 shots
-    // at p = 0.06 (1 round) 0.90x (1.14x); [[288]] R = 20 (one block per SM), 300 /
-    // 500 / 1,000 shots (1.2 / 2.1 / 4.1 rounds): 0.83x / 1.11x / 1.29x.
-    struct { int blocks, rounds2; } choices[] = {{4, 12}, {3, 12}, {2, 2}, {1, 3}};  // rounds in halves
-    for (const auto& c : choices) {
-        if ((size_t)c.blocks * L.total > 227 * 1024) continue;
-        const unsigned long long slots = (unsigned long long)c.blocks * sm_count * (kGroups * kShots);
-        if (2 * a.total_items < (unsigned long long)c.rounds2 * slots) continue;
-        const int threads = kMaxThreads / c.blocks / (32 * kGroups) * (32 * kGroups);
-        int per_sm = 0;
+    int blocks = 4, threads = 0, per_sm = 0;
+    for (;; --blocks) {
+        if (blocks > 1 && (size_t)blocks * L.total > 227 * 1024) continue;
+        threads = kMaxThreads / blocks / (32 * kGroups) * (32 * kGroups);
         const cudaError_t e = prepare_kernel(reinterpret_cast<const void*>(kern), threads, (size_t)L.total, &per_sm);
         if (e != cudaSuccess) return e;
-        const unsigned long long blocks = (a.total_items + kGroups * kShots - 1) / (kGroups * kShots);
-        const unsigned grid = (unsigned)std::min<unsigned long long>((unsigned long long)per_sm * sm_count, blocks);
-        kern<<<grid, threads, L.total, s>>>(a);
-        *taken = true;
-        return cudaGetLastError();
+        if (per_sm >= blocks) break;  // what a block takes besides can leave room for one less
     }
-    return cudaSuccess;
+    const unsigned long long items = (a.total_items + kGroups * kShots - 1) / (kGroups * kShots);
+    kern<<<(unsigned)std::min<unsigned long long>((unsigned long long)per_sm * sm_count, items), threads, L.total, s>>>(a);
+    return cudaGetLastError();
 }
 
 template <int DC>
-cudaError_t launch_width(const DecodeArgs& a, cudaStream_t s, int sm_count, bool* taken) {
+cudaError_t launch_width(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     const bool reg = a.B.regular != 0;
     if (a.rule == MBBP_RULE_NMS)
-        return reg ? launch_t<DC, MBBP_RULE_NMS, true>(a, s, sm_count, taken)
-                   : launch_t<DC, MBBP_RULE_NMS, false>(a, s, sm_count, taken);
-    return reg ? launch_t<DC, MBBP_RULE_SP, true>(a, s, sm_count, taken)
-               : launch_t<DC, MBBP_RULE_SP, false>(a, s, sm_count, taken);
+        return reg ? launch_t<DC, MBBP_RULE_NMS, true>(a, s, sm_count)
+                   : launch_t<DC, MBBP_RULE_NMS, false>(a, s, sm_count);
+    return reg ? launch_t<DC, MBBP_RULE_SP, true>(a, s, sm_count)
+               : launch_t<DC, MBBP_RULE_SP, false>(a, s, sm_count);
 }
 
 }  // namespace
 
-cudaError_t launch_decode_serial_lanes(const DecodeArgs& a, cudaStream_t s, int sm_count, bool* taken) {
-    const DevBases& B = a.B;
-    *taken = false;
-    if (a.io.post || a.io.llr_stride != 0 || !B.edesc) return cudaSuccess;
-    if (serial_lanes_layout(B.DC, B.lsteps, B.m, B.n).total > kMaxDynamic) return cudaSuccess;
-    if (B.DC == 6) return launch_width<6>(a, s, sm_count, taken);
-    if (B.DC == 8) return launch_width<8>(a, s, sm_count, taken);
-    return cudaSuccess;
+cudaError_t launch_decode_serial_lanes(const DecodeArgs& args, cudaStream_t s, int sm_count, const unsigned int** flag) {
+    const DevBases& B = args.B;
+    *flag = nullptr;
+    const double rounds = (double)args.total_items / (32.0 * sm_count);
+    if (rounds < kMinRounds || args.io.post || args.io.llr_stride != 0 ||
+        serial_lanes_layout(B.DC, B.lsteps, B.m, B.n).total > kMaxDynamic)
+        return cudaMemsetAsync(args.rep_counter, 0, sizeof(unsigned int) * (size_t)B.R, s);
+    DecodeArgs a = args;
+    unsigned int* word = reinterpret_cast<unsigned int*>(a.counter);  // a work counter that this path does not use
+    a.lanes = word;
+    serial_route_kernel<<<1, kRouteThreads, 0, s>>>(a.io.synd, B.m, a.io.batch, B.R, min_density(a.rule, rounds), word,
+                                                    a.rep_counter);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    *flag = word;
+    return B.DC == 6 ? launch_width<6>(a, s, sm_count) : launch_width<8>(a, s, sm_count);
 }
 
 }  // namespace mbbp

@@ -1167,13 +1167,11 @@ mbbp_status decode_impl(const mbbp_bases* B, int batch, const uint8_t* syndromes
     a.total_items = (unsigned long long)batch * B->R;
     a.rep_counter = reinterpret_cast<unsigned int*>(a.counter + 1);
     cudaError_t e = cudaSuccess;
-    if (opt->schedule == MBBP_SCHEDULE_SERIAL) {
-        const size_t counter_bytes = sizeof(unsigned long long) + sizeof(unsigned int) * (size_t)B->R;
-        e = cudaMemsetAsync(a.counter, 0, counter_bytes, s);
-        if (e == cudaSuccess) e = launch_decode_serial(a, s, B->sm_count);
-    } else {
-        e = launch_decode(a, s, B->sm_count);  // clears the work counter where its launch pulls from it
-    }
+    // both clear the work counters where their launch pulls from them
+    if (opt->schedule == MBBP_SCHEDULE_SERIAL)
+        e = launch_decode_serial(a, s, B->sm_count);
+    else
+        e = launch_decode(a, s, B->sm_count);
     if (e != cudaSuccess) return cuda_fail(e, "mbbp_decode (BP)");
     FwsArgs f{};
     f.cand = a.io.cand;

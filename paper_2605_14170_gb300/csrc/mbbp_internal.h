@@ -187,6 +187,8 @@ struct DecodeArgs {
     unsigned long long* counter;
     unsigned long long total_items;
     unsigned int* rep_counter;  // [R] next shot of each representation (serial slot path)
+    const unsigned int* lanes;  // serial slot path: set on the device when the one-shot-per-lane kernel
+                                // takes the call (null: the warp-per-slot kernel does)
 };
 
 struct FwsArgs {
@@ -283,9 +285,10 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t s, int sm_count);
 cudaError_t launch_decode_serial(const DecodeArgs& a, cudaStream_t s, int sm_count);
 cudaError_t launch_decode_serial_generic(const DecodeArgs& a, cudaStream_t s, int sm_count);
 cudaError_t launch_decode_small(const DecodeArgs& a, cudaStream_t s, int sm_count);
-// One shot per lane (decode_serial_lanes.cu); *taken = false, nothing launched,
-// for calls that stay with the warp-per-slot kernel.
-cudaError_t launch_decode_serial_lanes(const DecodeArgs& a, cudaStream_t s, int sm_count, bool* taken);
+// One shot per lane (decode_serial_lanes.cu).  Clears the counters; *flag = the
+// word on the device that says whether this kernel takes the call, null when
+// it was not launched.
+cudaError_t launch_decode_serial_lanes(const DecodeArgs& a, cudaStream_t s, int sm_count, const unsigned int** flag);
 cudaError_t launch_fws(const FwsArgs& a, cudaStream_t s);
 // Device address of the fixed scratch array on the current device (looked up
 // on the first call per device).

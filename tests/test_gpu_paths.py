@@ -262,6 +262,74 @@ def test_serial_one_shot_per_lane_shared_memory_limit(size):
     _assert_exact({k: v[:16] for k, v in got.items()}, few)
 
 
+SERIAL_BLOCKS = {  # code, R: blocks of the one-shot-per-lane kernel that an SM holds
+    "bb72": (lambda: named_code("bb72").HZ, 64),                                # 4
+    "gb36w4": (lambda: gb_code(18, [0, 3, 11, 16], [1, 8, 12, 15]).HZ, 8),      # 4, width 8
+    "gb100": (lambda: gb_code(50, [0, 7, 31], [2, 19, 44]).HZ, 20),             # 3
+    "bb144": (lambda: named_code("bb144").HZ, 64),                              # 2
+    "irregular8": (lambda: _irregular(60, 120, 8, 6), 8),                       # 1, width 8
+}
+
+
+@pytest.mark.parametrize("rule,iters", [("nms", 0), ("nms", 9), ("sp", 9)])
+@pytest.mark.parametrize("code", sorted(SERIAL_BLOCKS))
+def test_serial_one_shot_per_lane_blocks(code, rule, iters):
+    """The one-shot-per-lane kernel at each number of blocks per SM, both
+    widths, irregular rows, and no iterations at all: 130,000 (shot,
+    representation) pairs of random syndromes, which the kernel takes (the
+    word behind the candidates says so).  Bit for bit as the warp-per-slot
+    kernel and, min-sum, for the first shots as the FP32 oracle."""
+    import torch
+    from paper_2605_14170_gb300 import mbbp
+    make, R = SERIAL_BLOCKS[code]
+    H = make()
+    n, shots = H.shape[1], 130_000 // R
+    e, _ = oracle.sample(SEED + 7, 0, shots, n, 0.4, "bsc")
+    s = oracle.syndrome(H, e)
+    s[:5] = 0  # halt at once
+    llr = np.random.default_rng(8).uniform(0.5, 2.0, n).astype(np.float32)
+    B = mbbp.mbbp_build_bases(H, R, SEED)
+    kw = dict(rule=mbbp.RULE_SP if rule == "sp" else mbbp.RULE_NMS, schedule=mbbp.SCHEDULE_SERIAL)
+    st = torch.from_numpy(s).cuda()
+    lanes, slots = (mbbp.decode(B, st, torch.from_numpy(x).cuda(), iters, 0.8, **kw)
+                    for x in (llr, np.tile(llr, (shots, 1))))
+    torch.cuda.synchronize()
+    word = (shots * R * ((n + 31) // 32) * 4 + 255) // 256 * 256
+    assert int(lanes["workspace"][word:word + 4].view(torch.int32)) == 1
+    for key in ("conv", "iters", "cand", "selected", "success", "e_hat"):
+        assert torch.equal(lanes[key], slots[key]), key
+    if rule == "nms":
+        got = {k: v[:32].cpu().numpy() for k, v in lanes.items() if k != "workspace"}
+        got["iters"], got["cand"] = got["iters"].view(np.uint16), mbbp.unpack_words(got["cand"], n)
+        _assert_exact(got, oracle.mbbp_decode(H, B.sets, s[:32], llr, iters, 0.8, precision="f32",
+                                              schedule=oracle.SCHEDULE_SERIAL))
+
+
+@pytest.mark.parametrize("p,rounds,lanes", [(0.004, 40, 0), (0.03, 20, 0), (0.08, 20, 1), (0.08, 12, 0)])
+def test_serial_route(p, rounds, lanes):
+    """The rule of the one-shot-per-lane kernel: at least 16 rounds of 32 items
+    per SM and rounds * density^2 >= 1 (syndrome densities 0.02, 0.16 and
+    0.32), decided on the device; the result is the oracle's either way."""
+    import torch
+    from paper_2605_14170_gb300 import mbbp
+    H, R, n = named_code("bb72").HZ, 64, 72
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    shots = 32 * sms * rounds // R
+    e, _ = oracle.sample(SEED + 8, 0, shots, n, p, "bsc")
+    s = oracle.syndrome(H, e)
+    llr = channel_llr(n, p).astype(np.float32)
+    B = mbbp.mbbp_build_bases(H, R, SEED)
+    out = mbbp.decode(B, torch.from_numpy(s).cuda(), torch.from_numpy(llr).cuda(), 20, 0.8,
+                      schedule=mbbp.SCHEDULE_SERIAL)
+    torch.cuda.synchronize()
+    word = (shots * R * 3 * 4 + 255) // 256 * 256
+    if rounds >= 16:
+        assert int(out["workspace"][word:word + 4].view(torch.int32)) == lanes
+    ref = oracle.mbbp_decode(H, B.sets, s[:100], llr, 20, 0.8, precision="f32", schedule=oracle.SCHEDULE_SERIAL)
+    for key, rkey in (("e_hat", "ehat"), ("conv", "conv"), ("success", "success"), ("selected", "selected")):
+        assert np.array_equal(out[key][:100].cpu().numpy(), ref[rkey]), key
+
+
 @pytest.mark.parametrize("R", [1, 4, 5, 8, 9, 16, 17, 32, 33, 64])
 def test_selection_widths(R):
     """Frequency-weighted selection with 4, 8, 16 or 32 lanes per shot (R up to
