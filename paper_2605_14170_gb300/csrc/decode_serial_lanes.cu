@@ -127,31 +127,33 @@ __device__ __forceinline__ void lane_posts(int& st, int nw, const int* cend, con
     if constexpr (D < DC) lane_posts<D + 1, DC>(st, nw, cend, ms, var, ew);
 }
 
-// Which of the two serial kernels takes a call.  A shot that halts here makes
-// its block refill a slot and the last shots of a representation run at this
-// kernel's pace per iteration, 2-3 times slower than a warp per slot; both are
-// small beside the iterations of a long batch whose shots take several.  How
-// many they take shows in the syndromes, which are on the device: so one block
-// counts the ones of 128 of them, spread over the batch, sets *flag, and of the
-// two kernels launched after it the other returns at once.  It also clears the
-// counters, so a call pays for one empty launch more (AAA).
+// Which of the two serial kernels takes a call.  A shot that halts in this one
+// makes its group refill a slot, and the last shots of a representation run at
+// its slower pace per iteration (one of 32 shots of a block against one of at
+// most 4 of a warp); both are small only beside the iterations of a long batch
+// of shots that take several.  How many they take shows in the syndromes, which
+// are on the device.  So one block counts the ones of 128 syndromes spread over
+// the batch and sets *flag; of the two kernels launched after it the other
+// returns at once.  It clears the shot counters too, in place of a memset.  A
+// call that stays with the warp-per-slot kernel pays 3 to 8 us for both launches:
+// [[72]] R = 4, 20,000 shots at p = 0.001 87 us, 82 without them.
 //
-// min-sum: rounds * density^2 >= 1 and density >= 0.1, a round being 32 items
-// (one block's slots) per SM.  Measured against the warp-per-slot kernel
-// (13 codes of length 60 to 288, rows of weight 2 to 8, R = 4 to 20, error
-// rates 0.001 to 0.2, alpha 0.625 and 0.875, 1 to 100 iterations): no point
-// that satisfies the rule is slower.  Worst and best of the codes with rows of
-// weight 6, 100 iterations, by density (0.056: 1%, 0.11: 2%, 0.20: 4%, 0.27: 6%,
-// 0.32: 8% errors) and rounds:
-//              4          16         32         96
-//   0.056      -       0.68-1.12  0.85-1.1  0.86-1.16
-//   0.11       -       0.73-1.12  0.84-1.29  1.04-1.83
-//   0.20       -       0.90-1.82  1.03-2.08  1.18-2.51
-//   0.27   0.77-1.33   1.06-2.19  1.21-2.56  -
-//   0.32   0.88-1.52   1.22-2.59  1.28-2.85  -
-// Sum-product shots take longer in one lane: rounds * density^2 >= 4 and
-// density >= 0.2 (0.2, 64 rounds: 0.97-2.0; 0.32, 16 rounds: 0.91-2.2, 64:
-// 1.10-2.4).
+// Min-sum: rounds * density^2 >= 1 and density >= 0.1, a round being 32 items
+// per SM.  Times as fast as the warp-per-slot kernel (nine or ten codes with rows
+// of weight 6, length 60 to 288, R = 4 to 20, alpha 0.875, 100 iterations;
+// slowest to fastest code), by error rate, density and rounds:
+//      p    density      4         16         32         96
+//   0.001   0.006   0.56-1.99  0.53-1.85      -      0.48-0.97
+//   0.01    0.056   0.73-1.12  0.77-1.12      -      0.88-1.16
+//   0.02    0.11    0.61-1.02  0.71-1.12  0.84-1.29  1.04-1.85
+//   0.04    0.20    0.65-1.14  0.90-1.82  1.03-2.08  1.17-2.52
+//   0.06    0.27    0.77-1.33  1.03-2.19  1.21-2.56  1.47-2.90
+//   0.08    0.32    0.88-1.52  1.22-2.59  1.28-2.85      -
+// Rows of weight 8, irregular rows, alpha 0.625 and limits of 1 to 50 iterations
+// lie higher at the same density.  1.03 is the least of all measured points that
+// satisfy the rule.  Sum-product takes longer in one lane: rounds * density^2 >=
+// 6 and density >= 0.2 (0.20, 64 rounds: 0.97-2.04; 0.32, 16: 0.91-2.00, 64:
+// 1.10-2.44).
 constexpr int kRouteShots = 128;
 constexpr int kRouteThreads = 1024;
 constexpr int kMinRounds = 16;
