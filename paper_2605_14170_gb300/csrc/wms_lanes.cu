@@ -13,10 +13,10 @@
 // uncoalesced float atomic per parameter and shot; these 49 and 113.
 // Messages live in shared memory, the adjoint's recomputed states in the
 // workspace (they stay in L2).  Issue slots are 60-65% busy; the rest is
-// latency: barriers between the passes and the state loads.  24 warps per SM
-// at 80 registers: fewer warps with more registers, more with spills, 32 shots
-// per block, wider parameter or record loads and a prefetch of the next row's
-// state all measured slower or the same.
+// latency: barriers between the passes and the state loads.  At width 6, 24
+// warps per SM at 80 registers: fewer warps with more registers, more with
+// spills, 32 shots per block, wider parameter or record loads and a prefetch of
+// the next row's state all measured slower or the same.
 //
 // [[144,12,12]] R = 8, T = 25, checkpoints every 5, batch 4096: forward 0.93 ->
 // 0.72 ms, backward 4.58 -> 1.98 ms (0.74 and 2.15 before the warp's index was
@@ -33,6 +33,15 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kLaneThreads = 768;  // largest block
+// Threads of the adjoint by kernel width: a row's edges are in registers
+// throughout, and with 80 of them (768 threads) width 8 spills 88 to 112 bytes
+// and width 12 408 to 424; with these 8 to 24 and 148 to 168 are left.  A step at
+// T = 20, checkpoints every 5, 768 -> these: width 8 (length 96, rows of 8,
+// R = 4, batch 300) 0.234 -> 0.213 ms, width 12 (length 96, rows of 10) 0.377 ->
+// 0.306 ms; batch 2000, R = 8 1.104 -> 1.053 and 2.108 -> 1.919.  512 and 384:
+// 0.207, 0.315; 1.143, 2.354 (12 warps per SM with two blocks of 6).
+template <int DC>
+constexpr int kBackwardThreads = DC == 12 ? 512 : (DC == 8 ? 640 : kLaneThreads);
 constexpr int kLaneRows = 2;       // rows (or variables) of a warp step
 constexpr int kLaneShots = 32 / kLaneRows;
 
@@ -377,7 +386,7 @@ __global__ void __launch_bounds__(kLaneThreads, 1) wms_forward_lanes_kernel(cons
 }
 
 template <int DC, bool REG>
-__global__ void __launch_bounds__(kLaneThreads, 1) wms_backward_lanes_kernel(const WmsArgs a, int batch, int blocks) {
+__global__ void __launch_bounds__(kBackwardThreads<DC>, 1) wms_backward_lanes_kernel(const WmsArgs a, int batch, int blocks) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int cls[48];
     __shared__ int s_item;
@@ -573,12 +582,13 @@ cudaError_t launch_lanes(const WmsArgs& a, int batch, bool backward, cudaStream_
                                        : reinterpret_cast<const void*>(wms_backward_lanes_kernel<DC, false>))
                                 : (reg ? reinterpret_cast<const void*>(wms_forward_lanes_kernel<DC, true>)
                                        : reinterpret_cast<const void*>(wms_forward_lanes_kernel<DC, false>));
-    // 24 warps per SM (80 registers): two blocks of 12 when their shared
-    // memory fits twice and there is work for both, else one of 24
-    int threads = kLaneThreads / 2, per_sm = 0;
+    // all warps that registers allow: two blocks of half of them when their
+    // shared memory fits twice and there is work for both, else one
+    const int most = backward ? kBackwardThreads<DC> : kLaneThreads;
+    int threads = most / 2, per_sm = 0;
     cudaError_t e = prepare_kernel(kern, threads, L.total, &per_sm);
     if (e == cudaSuccess && (per_sm < 2 || wms_lanes_grid(a.B, batch, sm_count) <= (size_t)sm_count)) {
-        threads = kLaneThreads;
+        threads = most;
         e = prepare_kernel(kern, threads, L.total, &per_sm);
     }
     if (e != cudaSuccess) return e;
@@ -594,8 +604,9 @@ cudaError_t launch_lanes(const WmsArgs& a, int batch, bool backward, cudaStream_
 bool wms_lanes_fit(const DevBases& B, int batch) {
     // From 256 (shot, representation) pairs on: 64 shots at R = 2 of
     // [[144,12,12]] took 0.284 ms a step here and 0.276 ms warp per shot, 64 at
-    // R = 8 0.284 and 0.322 ms.  The block's two message arrays must fit shared
-    // memory (the length-882 code's do not).
+    // R = 8 0.284 and 0.322 ms; 128 at R = 2 of codes of length 96 with rows of 8
+    // and 10 (T = 20) 0.213 and 0.260, 0.305 and 0.362.  The block's two message
+    // arrays must fit shared memory (the length-882 code's do not).
     const long long blocks = ((long long)batch + kLaneShots - 1) / kLaneShots;
     return (long long)batch * B.R >= 256 && blocks * B.R <= INT_MAX / 2 &&
            lanes_layout(B.DC, B.MP, B.n).total <= 226 * 1024 + 256;  // and 256 static
