@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <set>
 #include <string>
@@ -546,8 +547,7 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
     if ((long long)K * MP > MBBP_MAX_SLOTS) return fail(MBBP_E_TOO_LARGE, "too many edge slots");
     const int mpad = round_up(m, 32), W = words_for(n);
 
-    mbbp_bases* B = new (std::nothrow) mbbp_bases();
-    if (!B) return fail(MBBP_E_NOMEM, "host allocation failed");
+    std::unique_ptr<mbbp_bases> B(new mbbp_bases());
     B->m = m; B->n = n; B->R = R; B->K = K; B->DV = dv; B->MP = MP; B->mpad = mpad;
     B->W = W; B->regular = (regular && dc == K) ? 1 : 0;  // every row fills the kernel width
     B->H.assign(H, H + (size_t)m * n);
@@ -600,48 +600,60 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
         const int anneal = 20000;
         const int nth = std::max(1, std::min(R, (int)std::thread::hardware_concurrency()));
         std::atomic<int> next{0};
+        std::atomic<bool> no_memory{false};
+        auto layout = [&](int t) {
+            RepLayout& L = layouts[t];
+            const int M = m + set_ptr[t + 1] - set_ptr[t];
+            L.src.resize(M);
+            for (int r = 0; r < M; ++r) L.src[r] = r < m ? r : set_rows[set_ptr[t] + (r - m)];
+            // Serial schedule: rows go, in row order, into the first layer
+            // holding none of their variables.
+            std::vector<std::vector<uint8_t>> layer_vars;
+            std::vector<int> count;
+            std::vector<std::vector<int>> rc(M);
+            L.layer_of.resize(M);
+            L.idx_in.resize(M);
+            for (int r = 0; r < M; ++r) {
+                rc[r] = g.rcols[L.src[r]];
+                size_t y = 0;
+                for (; y < layer_vars.size(); ++y) {
+                    bool clash = false;
+                    for (int v : rc[r]) clash = clash || layer_vars[y][v];
+                    if (!clash) break;
+                }
+                if (y == layer_vars.size()) {
+                    layer_vars.emplace_back(n, 0);
+                    count.push_back(0);
+                }
+                for (int v : rc[r]) layer_vars[y][v] = 1;
+                L.layer_of[r] = (int)y;
+                L.idx_in[r] = count[y]++;
+            }
+            L.layers = (int)layer_vars.size();
+            if (chunked) {
+                const int CS = serial_bp::shots_per_warp(K, MP, mpad, n);
+                L.sp = serial_positions(rc, L.layer_of, L.idx_in, CS, K, n, 0xBA4Cull + (uint64_t)t);
+            }
+            L.generic = bank_layout(g, L.src, n, MP, 0x6E4Eull + (uint64_t)t, false, anneal);
+            if (shape) L.small = bank_layout(g, L.src, n, MP, 0x5EEDull + (uint64_t)t, true, 1000000);
+        };
         auto worker = [&]() {
-            for (int t = next++; t < R; t = next++) {
-                RepLayout& L = layouts[t];
-                const int M = m + set_ptr[t + 1] - set_ptr[t];
-                L.src.resize(M);
-                for (int r = 0; r < M; ++r) L.src[r] = r < m ? r : set_rows[set_ptr[t] + (r - m)];
-                // Serial schedule: rows go, in row order, into the first layer
-                // holding none of their variables.
-                std::vector<std::vector<uint8_t>> layer_vars;
-                std::vector<int> count;
-                std::vector<std::vector<int>> rc(M);
-                L.layer_of.resize(M);
-                L.idx_in.resize(M);
-                for (int r = 0; r < M; ++r) {
-                    rc[r] = g.rcols[L.src[r]];
-                    size_t y = 0;
-                    for (; y < layer_vars.size(); ++y) {
-                        bool clash = false;
-                        for (int v : rc[r]) clash = clash || layer_vars[y][v];
-                        if (!clash) break;
-                    }
-                    if (y == layer_vars.size()) {
-                        layer_vars.emplace_back(n, 0);
-                        count.push_back(0);
-                    }
-                    for (int v : rc[r]) layer_vars[y][v] = 1;
-                    L.layer_of[r] = (int)y;
-                    L.idx_in[r] = count[y]++;
-                }
-                L.layers = (int)layer_vars.size();
-                if (chunked) {
-                    const int CS = serial_bp::shots_per_warp(K, MP, mpad, n);
-                    L.sp = serial_positions(rc, L.layer_of, L.idx_in, CS, K, n, 0xBA4Cull + (uint64_t)t);
-                }
-                L.generic = bank_layout(g, L.src, n, MP, 0x6E4Eull + (uint64_t)t, false, anneal);
-                if (shape) L.small = bank_layout(g, L.src, n, MP, 0x5EEDull + (uint64_t)t, true, 1000000);
+            try {
+                for (int t = next++; t < R && !no_memory; t = next++) layout(t);
+            } catch (const std::bad_alloc&) {
+                no_memory = true;
             }
         };
         std::vector<std::thread> pool;
-        for (int i = 1; i < nth; ++i) pool.emplace_back(worker);
+        try {
+            pool.reserve(nth);
+            for (int i = 1; i < nth; ++i) pool.emplace_back(worker);
+        } catch (const std::exception&) {
+            // no further thread can start: those that did and this one do the work
+        }
         worker();
         for (auto& th : pool) th.join();
+        if (no_memory) return fail(MBBP_E_NOMEM, "out of memory");
     }
     auto slot_of = [&](int pos, int j) { return (pos >> 5) * (32 * K) + 32 * j + (pos & 31); };
     std::vector<uint16_t> lrows16((size_t)R * MP, 0);
@@ -826,10 +838,7 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
     cudaError_t e = cudaGetDevice(&B->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&B->sm_count, cudaDevAttrMultiProcessorCount, B->device);
     if (e == cudaSuccess) e = cudaMalloc(&B->dmem, total);
-    if (e != cudaSuccess) {
-        delete B;
-        return cuda_fail(e, "mbbp_build_bases");
-    }
+    if (e != cudaSuccess) return cuda_fail(e, "mbbp_build_bases");
     char* base = static_cast<char*>(B->dmem);
     struct Copy { size_t off; const void* src; size_t bytes; } copies[] = {
         {o_rowinfo, rowinfo.data(), rowinfo.size() * 4},
@@ -858,7 +867,6 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
         e = cudaMemcpy(base + c.off, c.src, c.bytes, cudaMemcpyHostToDevice);
         if (e != cudaSuccess) {
             cudaFree(B->dmem);
-            delete B;
             return cuda_fail(e, "mbbp_build_bases copy");
         }
     }
@@ -890,8 +898,19 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
     d.lpos = chunked ? reinterpret_cast<const uint16_t*>(base + o_lpos) : nullptr;
     d.lsteps = lsteps;
     d.rinfo_s = chunked ? reinterpret_cast<const uint32_t*>(base + o_rinfo_s) : nullptr;
-    *out = B;
+    *out = B.release();
     return MBBP_OK;
+}
+
+// build(), with a failed host allocation as a status: nothing is thrown
+// through the C interface.
+template <class F>
+mbbp_status no_throw(F&& build) {
+    try {
+        return build();
+    } catch (const std::bad_alloc&) {
+        return fail(MBBP_E_NOMEM, "out of memory");  // short enough not to allocate
+    }
 }
 
 mbbp_status check_device(int device) {
@@ -984,17 +1003,19 @@ mbbp_status mbbp_build_bases(const uint8_t* H, int m, int n, int R, uint64_t see
                              mbbp_bases** out) {
     if (out) *out = nullptr;
     if (R < 1 || R > MBBP_MAX_R) return fail(MBBP_E_INVALID, "R must be in [1, 64]");
-    Tanner g;
-    if (mbbp_status st = make_tanner(H, m, n, g)) return st;
-    std::vector<int32_t> ptr, rows;
-    if (mbbp_status st = collect_impl(g, R, seed, ptr, rows)) return st;
-    return build_impl(H, m, n, R, ptr.data(), rows.data(), out);
+    return no_throw([&]() -> mbbp_status {
+        Tanner g;
+        if (mbbp_status st = make_tanner(H, m, n, g)) return st;
+        std::vector<int32_t> ptr, rows;
+        if (mbbp_status st = collect_impl(g, R, seed, ptr, rows)) return st;
+        return build_impl(H, m, n, R, ptr.data(), rows.data(), out);
+    });
 }
 
 mbbp_status mbbp_build_bases_from_sets(const uint8_t* H, int m, int n, int R,
                                        const int32_t* set_ptr, const int32_t* set_rows,
                                        mbbp_bases** out) {
-    return build_impl(H, m, n, R, set_ptr, set_rows, out);
+    return no_throw([&]() { return build_impl(H, m, n, R, set_ptr, set_rows, out); });
 }
 
 mbbp_status mbbp_bases_info(const mbbp_bases* B, int32_t* m, int32_t* n, int32_t* R,
