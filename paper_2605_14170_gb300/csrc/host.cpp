@@ -301,6 +301,7 @@ BankLayout bank_layout(const Tanner& g, const std::vector<int>& src, int n, int 
             const int r = (int)(rnd() % M);
             const auto& cols = g.rcols[src[r]];
             const int d = (int)cols.size();
+            if (d == 0) continue;
             const int ja = (int)(rnd() % d), jb = (int)(rnd() % d);
             if (ja == jb) continue;
             const int ca = cell(cols[ja], ei[r][ja]), cb = cell(cols[jb], ei[r][jb]);

@@ -72,6 +72,24 @@ def test_generic_flooding_variants(code, post):
     _assert_exact(got, oracle.mbbp_decode(H, B.sets, s, llr, 40, 0.7, precision="f32"))
 
 
+@pytest.mark.parametrize("schedule", ["flooding", "serial"])
+@pytest.mark.parametrize("code", ["bb72", "irregular"])
+def test_empty_row(code, schedule):
+    """A matrix with a row without entries, in H and in a repeated set."""
+    from paper_2605_14170_gb300 import mbbp
+    H = (named_code("bb72").HZ if code == "bb72" else CODES[code]()).copy()
+    H[5] = 0
+    sets, n = [[0], [1, 5, 9], [2, 3]], H.shape[1]
+    e, _ = oracle.sample(SEED + 9, 0, 33, n, 0.04, "bsc")
+    s = oracle.syndrome(H, e)
+    llr = channel_llr(n, 0.04).astype(np.float32)
+    B = mbbp.mbbp_build_bases_from_sets(H, sets)
+    sched = (mbbp.SCHEDULE_SERIAL, oracle.SCHEDULE_SERIAL) if schedule == "serial" else (mbbp.SCHEDULE_FLOODING,
+                                                                                       oracle.SCHEDULE_FLOODING)
+    got = _decode(B, s, llr, 20, 0.7, schedule=sched[0])
+    _assert_exact(got, oracle.mbbp_decode(H, sets, s, llr, 20, 0.7, precision="f32", schedule=sched[1]))
+
+
 @pytest.mark.parametrize("ckpt,all_iters", [(1, True), (3, False), (7, True)])
 @pytest.mark.parametrize("code", ["bb72", "gb90w4", "gb78w5", "irregular"])
 def test_wms_training_one_shot_per_lane(code, ckpt, all_iters):

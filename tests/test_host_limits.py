@@ -1,7 +1,8 @@
-"""Building a handle where the host has no more threads or memory: a status,
-not the end of the process.  Run in a process of its own under an address-space
-limit, in which no thread's stack fits; without a GPU the build ends at its
-first CUDA call, behind the host's work."""
+"""Building a handle where the host has no more threads or memory, or for a
+matrix with an empty row: a status, not the end of the process.  Each in a
+process of its own, the first under an address-space limit in which no thread's
+stack fits; without a GPU the build ends at its first CUDA call, behind the
+host's work."""
 import subprocess
 import sys
 
@@ -53,3 +54,14 @@ def test_build_without_memory(code, R):
     far as the first did."""
     first, second, third = _run(code, R, 0)
     assert second == 5 and third == first
+
+
+def test_build_with_an_empty_row():
+    """A row of H without entries (a small code: its layout search swaps the
+    edges of a row)."""
+    program = PROGRAM.split("first =")[0] + "H[5] = 0\nprint(build(), build(named_code('bb72').HZ, 4))"
+    r = subprocess.run([sys.executable, "-c", program, "bb72", "4", "0"], cwd=ROOT, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0, (r.returncode, r.stderr[-2000:])
+    with_empty, without = (int(x) for x in r.stdout.split())
+    assert with_empty == without
