@@ -1560,6 +1560,7 @@ WmsWorkspace wms_workspace(const mbbp_bases* B, int batch, int T, int ckpt, bool
 
 size_t mbbp_wms_workspace_size(const mbbp_bases* B, int batch, int T, int ckpt) {
     if (!B || batch < 0 || T < 1 || ckpt < 1) return 0;
+    ckpt = std::min(ckpt, T);  // no segment is longer
     // the one-shot-per-lane kernels take shared LLRs only, so that the LLR
     // stride, which this size does not know, decides between the two
     const size_t base = wms_workspace(B, batch, T, ckpt, false).total;
@@ -1573,6 +1574,7 @@ mbbp_status mbbp_wms_forward(const mbbp_bases* B, int batch, const uint8_t* synd
                              void* workspace, size_t workspace_bytes, void* stream) {
     if (mbbp_status st = wms_check(B, batch, T, ckpt)) return st;
     if (batch == 0) return MBBP_OK;
+    ckpt = std::min(ckpt, T);  // no segment is longer
     if (!syndromes || !llr || !w || !g || !posterior || !workspace)
         return fail(MBBP_E_INVALID, "mbbp_wms_forward: NULL buffer");
     if (loss && !etrue) return fail(MBBP_E_INVALID, "loss needs etrue");
@@ -1612,6 +1614,7 @@ mbbp_status mbbp_wms_backward(const mbbp_bases* B, int batch, const uint8_t* syn
                               float* gg, void* workspace, size_t workspace_bytes, void* stream) {
     if (mbbp_status st = wms_check(B, batch, T, ckpt)) return st;
     if (batch == 0) return MBBP_OK;
+    ckpt = std::min(ckpt, T);  // no segment is longer
     if (!syndromes || !llr || !w || !g || !etrue || !posterior || !gw || !gg || !workspace)
         return fail(MBBP_E_INVALID, "mbbp_wms_backward: NULL buffer");
     if (llr_stride != 0 && llr_stride < B->n) return fail(MBBP_E_INVALID, "llr_stride must be 0 or >= n");

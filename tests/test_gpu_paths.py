@@ -173,6 +173,36 @@ def test_wms_training_odd_variable_classes(code, ckpt, all_iters):
         assert np.linalg.norm(got.double().cpu().numpy() - r) <= 1e-3 * np.linalg.norm(r)
 
 
+@pytest.mark.parametrize("batch", [20, 300])
+def test_wms_checkpoint_interval_beyond_T(batch):
+    """A checkpoint interval longer than T needs no more workspace than T
+    itself and gives the same gradients (to the order of their sums, as
+    above), with the kernels of one shot per lane (300 shots) and of one warp
+    per shot (20)."""
+    import torch
+    from paper_2605_14170_gb300 import mbbp
+    H, R, T, n = named_code("bb144").HZ, 8, 6, 144
+    e, _ = oracle.sample(SEED + 10, 0, batch, n, 0.05, "bsc")
+    s, et = torch.from_numpy(oracle.syndrome(H, e)).cuda(), torch.from_numpy(mbbp.pack_bits(e)).cuda()
+    B = mbbp.mbbp_build_bases(H, R, SEED)
+    w, g = mbbp.wms_params(B, T, alpha=0.7)
+    g += 0.1
+    mu = torch.from_numpy(np.random.default_rng(5).uniform(1.0, 3.5, n).astype(np.float32)).cuda()
+    assert mbbp.mbbp_wms_workspace_size(B, batch, T, 1000) == mbbp.mbbp_wms_workspace_size(B, batch, T, T)
+    res = []
+    for ckpt in (2, T, 1000):
+        post = torch.empty((batch, R, n), device="cuda")
+        gw, gg = torch.zeros_like(w), torch.zeros_like(g)
+        ws = torch.empty(mbbp.mbbp_wms_workspace_size(B, batch, T, ckpt), dtype=torch.uint8, device="cuda")
+        mbbp.mbbp_wms_forward(B, s, mu, T, w, g, ckpt, et, 1e-3, post, None, ws, all_iters=True)
+        mbbp.mbbp_wms_backward(B, s, mu, T, w, g, ckpt, et, 1e-3, post, gw, gg, ws, all_iters=True)
+        torch.cuda.synchronize()
+        res.append([x.double() for x in (gw, gg)])
+    for other in res[1:]:
+        for a, b in zip(other, res[0]):
+            assert float(b.norm()) > 0 and float((a - b).norm()) <= 1e-4 * float(b.norm())
+
+
 @pytest.mark.parametrize("shots", [1, 3, 200, 1601])
 def test_small_code_run_lengths(shots):
     """The small-code kernel's runs of 8, 2 and 1 shots ([[72]], R = 64: the
