@@ -284,9 +284,11 @@ __device__ __forceinline__ void store_item_group(const ShotIO& io, unsigned long
 // variable positions likewise (gt: the thread's index in the group) and meet
 // on named barrier `bar` between passes; the arithmetic of every row and
 // variable is the same whatever G.  REG: every row fills the kernel width.
-// OUT: the call asks for posteriors (io.post) and / or the check messages of
-// every iteration (io.c2v; the last one run remains); without OUT the loops
-// carry no test for them.  Both are compiled apart because the passes are
+// OUT: kOutPosteriors: the call asks for posteriors (io.post); kOutAny: for the
+// check messages of every iteration (io.c2v; the last one run remains) and / or
+// posteriors; with kOutNone the loops carry no test for them.  Posteriors are
+// stored by position, coalesced, and go to their variables at the end of the
+// item.  REG and OUT are compiled apart because the passes are
 // bound by issue slots and the shared-memory path ([[288,12,18]]: 40
 // instructions per lane and edge update, the path 90% busy, 35% of its
 // wavefronts bank conflicts).  With the blocked slots, the bank-aware
@@ -294,8 +296,13 @@ __device__ __forceinline__ void store_item_group(const ShotIO& io, unsigned long
 // 8.10 -> 7.76 ms; length-882 code R = 64, 5,000 shots at p = 0.0333, 17.0 ->
 // 15.4 ms; a length-254 code with rows of weight 8, 3,001 shots, 282 -> 241
 // us; weighted min-sum decoding of 2,000 shots of the length-882 code 8.17 ->
-// 7.07 ms; training step on [[144,12,12]] R = 8 5.73 -> 5.55 ms.
-template <int DC, int DV, int RULE, bool REG, bool OUT, int G = 1>
+// 7.07 ms; training step on [[144,12,12]] R = 8 5.73 -> 5.55 ms.  With
+// posteriors, on the same codes, scattered to their variables in every iteration
+// by one body for all outputs and all rows -> this: R = 8, 5,000 shots 620 -> 521
+// us; R = 16, 1,000 shots 795 -> 683 us; 459 -> 421 us.
+constexpr int kOutNone = 0, kOutPosteriors = 1, kOutAny = 2;
+
+template <int DC, int DV, int RULE, bool REG, int OUT, int G = 1>
 __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, int shot, int b,
                                          unsigned char* area, const uint16_t* hcol, int bar = 0) {
     constexpr int GT = 32 * G;
@@ -341,7 +348,7 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
 #pragma unroll
             for (int i = 0; i < 6; ++i)
                 if (i < deg) msg_at(msg, packed_off(d, i)) = x;
-            if (OUT && io.post) io.post[item * n + v] = x;
+            if (OUT == kOutPosteriors || (OUT == kOutAny && io.post)) io.post[item * n + p] = x;
         }
     } else {
         for (int p = lane; p < n; p += GT) {
@@ -350,7 +357,7 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
             const float x = __fadd_rn(__ldg(llr + v), 0.0f);
             mu_s[p] = x;
             for (int i = 0; i < deg; ++i) msg[__ldg(B.vslot + d.x + i)] = x;
-            if (OUT && io.post) io.post[item * n + v] = x;
+            if (OUT == kOutPosteriors || (OUT == kOutAny && io.post)) io.post[item * n + p] = x;
         }
     }
     gsync<G>(bar);
@@ -395,7 +402,9 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
             const int r = lane + GT * k;
             if (r < Mb) {
                 const int deg = REG ? DC : (int)((__ldg(rinfo + r) >> 16) & 0xffu);
-                float* tr = (OUT && io.c2v) ? io.c2v + item * (unsigned long long)io.c2v_stride +
+                // (io.c2v is never null here; without the test the kernel measured 3 to
+                // 14% slower)
+                float* tr = (OUT == kOutAny && io.c2v) ? io.c2v + item * (unsigned long long)io.c2v_stride +
                                                   __ldg(B.rowptr + (size_t)b * MP + r)
                                             : nullptr;
                 check_row<DC, RULE, REG>(row, deg, (sb >> k) & 1u, io.alpha, tr);
@@ -414,7 +423,7 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
                 const int v = d.x & 0xffff, deg = (int)(d.x >> 16);
                 const float post = var_dispatch_packed(deg, msg, d, mu_s[p]);
                 eh[v] = (post < 0.f) ? 1 : 0;
-                if (OUT && io.post) io.post[item * n + v] = post;
+                if (OUT == kOutPosteriors || (OUT == kOutAny && io.post)) io.post[item * n + p] = post;
             }
         } else {
             uint2 dn = (lane < n) ? __ldg(vd + lane) : make_uint2(0u, 0u);
@@ -424,10 +433,16 @@ __device__ __forceinline__ void run_item(const DevBases& B, const ShotIO& io, in
                 const int v = d.y & 0xffff, deg = (int)(d.y >> 16);
                 const float post = var_dispatch<1, DV>(deg, msg, B.vslot + d.x, mu_s[p]);
                 eh[v] = (post < 0.f) ? 1 : 0;
-                if (OUT && io.post) io.post[item * n + v] = post;
+                if (OUT == kOutPosteriors || (OUT == kOutAny && io.post)) io.post[item * n + p] = post;
             }
         }
         gsync<G>(bar);
+    }
+    if (OUT == kOutPosteriors || (OUT == kOutAny && io.post)) {
+        float* post = io.post + item * n;
+        for (int p = lane; p < n; p += GT) mu_s[__ldg(&vd[p].y) & 0xffffu] = post[p];
+        gsync<G>(bar);
+        for (int v = lane; v < n; v += GT) post[v] = mu_s[v];
     }
     // candidate e_t (bit-packed), convergence flag, iterations
     if constexpr (G == 1)
@@ -561,17 +576,20 @@ __device__ __forceinline__ void run_item_serial(const DevBases& B, const ShotIO&
     __syncwarp();
 }
 
-// Dispatch on the kernel width of a representation set and on its rows.
+// Dispatch on the kernel width of a representation set and, at width 6, on its
+// rows.  At widths 8 and 12 every row loads its degree (two codes of length 120
+// and 180 with rows of 8, R = 8, 4,000 shots each: 508 us; 552 with the slots in
+// rows of MP and no such load; lengths 120 and 160, rows of 10 and 12: 1007, 1072).
 template <int RULE>
 __device__ __forceinline__ void run_item_any(const DevBases& B, const ShotIO& io, int shot, int b,
                                              unsigned char* area, const uint16_t* hcol) {
     if (B.DC == 6) {
-        if (B.regular) run_item<6, 6, RULE, true, false>(B, io, shot, b, area, hcol);
-        else run_item<6, 6, RULE, false, false>(B, io, shot, b, area, hcol);
+        if (B.regular) run_item<6, 6, RULE, true, kOutNone>(B, io, shot, b, area, hcol);
+        else run_item<6, 6, RULE, false, kOutNone>(B, io, shot, b, area, hcol);
     } else if (B.DC == 8) {
-        run_item<8, 8, RULE, false, false>(B, io, shot, b, area, hcol);
+        run_item<8, 8, RULE, false, kOutNone>(B, io, shot, b, area, hcol);
     } else {
-        run_item<12, 12, RULE, false, false>(B, io, shot, b, area, hcol);
+        run_item<12, 12, RULE, false, kOutNone>(B, io, shot, b, area, hcol);
     }
 }
 

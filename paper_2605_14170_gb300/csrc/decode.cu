@@ -33,7 +33,7 @@ constexpr int kGenericWideWarps = 16;
 // for codes whose per-item shared memory, not registers, limits the resident
 // warps: the same shared memory then holds G times the warps).  Group g of
 // the block uses named barrier 1 + g (at most 8 groups: ids 1..8).
-template <int DC, int DV, int RULE, int MAXW, bool REG, bool OUT, int G>
+template <int DC, int DV, int RULE, int MAXW, bool REG, int OUT, int G>
 __global__ void __launch_bounds__(MAXW * 32)
 decode_kernel(const DecodeArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -297,7 +297,7 @@ cudaError_t launch_serial_t(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     return cudaGetLastError();
 }
 
-template <int K, int RULE, bool REG, bool OUT, int G>
+template <int K, int RULE, bool REG, int OUT, int G>
 cudaError_t launch_decode_g(const DecodeArgs& a, int cls, int warps, int per_sm, size_t smem, cudaStream_t s,
                             int sm_count) {
     const unsigned long long groups = (unsigned long long)(warps / G);
@@ -312,7 +312,7 @@ cudaError_t launch_decode_g(const DecodeArgs& a, int cls, int warps, int per_sm,
     return cudaGetLastError();
 }
 
-template <int K, int RULE, bool REG, bool OUT>
+template <int K, int RULE, bool REG, int OUT>
 cudaError_t launch_decode_t(const DecodeArgs& a, cudaStream_t s, int sm_count) {
     // Launch shapes: (block class, warps per item G in {1, 2, 4}).  The narrow
     // class runs blocks of up to 8 warps, the wide class up to 16 (compiled
@@ -367,11 +367,17 @@ cudaError_t launch_decode_t(const DecodeArgs& a, cudaStream_t s, int sm_count) {
 
 template <int K, int RULE>
 cudaError_t launch_decode_k(const DecodeArgs& a, cudaStream_t s, int sm_count) {
-    // posteriors and the message trace take a kernel of their own, as do
-    // codes whose rows all fill the kernel width
-    if (a.io.c2v || a.io.post) return launch_decode_t<K, RULE, false, true>(a, s, sm_count);
-    if (a.B.regular) return launch_decode_t<K, RULE, true, false>(a, s, sm_count);
-    return launch_decode_t<K, RULE, false, false>(a, s, sm_count);
+    // calls for posteriors take kernels of their own, as do codes whose rows all
+    // fill the kernel width; message traces (a diagnosis) take one for all
+    // rows: with full rows apart it measured slower on codes of length 882 and 400
+    // (1.04 -> 1.14 ms, 0.66 -> 0.68) than it gained on [[288]] (0.75 -> 0.73)
+    using namespace generic_bp;
+    if (a.io.c2v) return launch_decode_t<K, RULE, false, kOutAny>(a, s, sm_count);
+    if (a.io.post)
+        return a.B.regular ? launch_decode_t<K, RULE, true, kOutPosteriors>(a, s, sm_count)
+                           : launch_decode_t<K, RULE, false, kOutPosteriors>(a, s, sm_count);
+    return a.B.regular ? launch_decode_t<K, RULE, true, kOutNone>(a, s, sm_count)
+                       : launch_decode_t<K, RULE, false, kOutNone>(a, s, sm_count);
 }
 
 }  // namespace

@@ -72,6 +72,29 @@ def test_generic_flooding_variants(code, post):
     _assert_exact(got, oracle.mbbp_decode(H, B.sets, s, llr, 40, 0.7, precision="f32"))
 
 
+@pytest.mark.parametrize("iters", [0, 1, 40])
+@pytest.mark.parametrize("code", sorted(CODES))
+def test_generic_posteriors(code, iters):
+    """Posteriors of the generic flooding kernels, which hold them by position
+    until an item ends, by variable as the FP32 oracle has them: bit for bit,
+    alone and together with the message trace."""
+    import torch
+    from paper_2605_14170_gb300 import mbbp
+    H = CODES[code]()
+    n, R = H.shape[1], 3
+    e, _ = oracle.sample(SEED + 11, 0, 17, n, 0.04, "bsc")
+    s = oracle.syndrome(H, e)
+    llr = np.random.default_rng(12).uniform(1.0, 3.0, n).astype(np.float32)
+    B = mbbp.mbbp_build_bases(H, R, SEED)
+    ref = np.stack([[oracle.bp(np.vstack([H, H[rows]]), np.concatenate([x, x[rows]]), llr, iters, 0.7,
+                               precision="f32")["post"] for rows in B.sets] for x in s])
+    for trace in (False, True):
+        out = mbbp.decode(B, torch.from_numpy(s).cuda(), torch.from_numpy(llr).cuda(), iters, 0.7,
+                          want_posterior=True, want_c2v=trace)
+        torch.cuda.synchronize()
+        assert np.array_equal(out["posterior"].cpu().numpy(), ref), trace
+
+
 @pytest.mark.parametrize("schedule", ["flooding", "serial"])
 @pytest.mark.parametrize("code", ["bb72", "irregular"])
 def test_empty_row(code, schedule):
