@@ -478,9 +478,9 @@ __device__ __forceinline__ void run_item_serial(const DevBases& B, const ShotIO&
     const int row_steps = MP >> 5;
     const int orow_steps = mpad >> 5;
     const unsigned long long item = (unsigned long long)shot * R + b;
-    const uint32_t* rinfo = B.rowinfo + (size_t)b * MP;
-    const uint2* vd = B.vdesc + (size_t)b * n;
-    const uint16_t* lrows = B.lrows + (size_t)b * MP;
+    const uint32_t* rinfo = B.rinfo_s + (size_t)b * MP;
+    const uint2* vd = B.vdesc_s + (size_t)b * n;
+    const uint16_t* lrows = B.lpos + (size_t)b * MP;
     const uint16_t* lptr = B.lptr + (size_t)b * (MP + 1);
     const uint2* ev = B.evar + (size_t)b * DC * MP;
     const int nl = __ldg(B.nlayers + b);
@@ -544,7 +544,7 @@ __device__ __forceinline__ void run_item_serial(const DevBases& B, const ShotIO&
                     q[j] = MBBP_LMAX;
                     if (j < deg) {
                         const int slot = row_slot<DC>(r) + 32 * j;
-                        const uint2 e = __ldg(ev + slot);
+                        const uint2 e = __ldg(ev + row_slot<DC>(idx) + 32 * j);
                         const int dv = (int)(e.y >> 16);
                         float x = mu_s[e.y & 0xffffu];
 #pragma unroll

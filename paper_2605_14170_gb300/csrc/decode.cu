@@ -71,10 +71,15 @@ decode_kernel(const DecodeArgs a) {
     }
 }
 
-// The serial-schedule kernel: same work list as decode_kernel, one warp per
-// (shot, representation) item, run_item_serial per item.
+// The serial-schedule kernel of width 12: same work list as decode_kernel, one
+// warp per (shot, representation) item, run_item_serial per item.  A layer of
+// such a code has 4 to 12 rows and each row gathers up to 132 messages one after
+// another, so loads in flight bound it: with 40 registers, the compiler's own
+// choice, a length-120 code with rows of 10, R = 8, 2,000 shots at p = 0.03, 100
+// iterations, took 14.2 ms, with the 55 of this bound 11.1 (2 and 3 blocks: 10.9,
+// 11.3; but 20,000 shots at p = 0.0127 5.66 -> 5.63, 6.16, 5.60).
 template <int DC, int DV, int RULE>
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+__global__ void __launch_bounds__(kWarpsPerBlock * 32, 4)
 decode_serial_kernel(const DecodeArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     const DevBases& B = a.B;
@@ -453,17 +458,9 @@ cudaError_t launch_decode(const DecodeArgs& a, cudaStream_t s, int sm_count) {
 }
 
 cudaError_t launch_decode_serial_generic(const DecodeArgs& a, cudaStream_t s, int sm_count) {
-    const int K = a.B.DC;
-    if (a.rule == MBBP_RULE_NMS) {
-        if (K == 6) return launch_serial_t<6, MBBP_RULE_NMS>(a, s, sm_count);
-        if (K == 8) return launch_serial_t<8, MBBP_RULE_NMS>(a, s, sm_count);
-        if (K == 12) return launch_serial_t<12, MBBP_RULE_NMS>(a, s, sm_count);
-    } else {
-        if (K == 6) return launch_serial_t<6, MBBP_RULE_SP>(a, s, sm_count);
-        if (K == 8) return launch_serial_t<8, MBBP_RULE_SP>(a, s, sm_count);
-        if (K == 12) return launch_serial_t<12, MBBP_RULE_SP>(a, s, sm_count);
-    }
-    return cudaErrorInvalidValue;
+    if (a.B.DC != 12) return cudaErrorInvalidValue;  // widths 6 and 8: decode_serial.cu
+    return a.rule == MBBP_RULE_NMS ? launch_serial_t<12, MBBP_RULE_NMS>(a, s, sm_count)
+                                   : launch_serial_t<12, MBBP_RULE_SP>(a, s, sm_count);
 }
 
 cudaError_t launch_fws(const FwsArgs& a, cudaStream_t s) {

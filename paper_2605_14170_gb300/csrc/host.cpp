@@ -564,15 +564,16 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
     // dependent load
     std::vector<uint4> vdesc6(K == 6 ? (size_t)R * n : 0, make_uint4(0, 0, 0, 0));
     std::vector<int32_t> rows(R), edges(R);
-    std::vector<uint2> evar((size_t)R * K * MP, make_uint2(0, 0));
     // chunked serial path (widths 6 and 8): per-edge and per-variable slot
     // descriptors with byte offsets, padded with the -0.0f slot
     const bool chunked = (K == 6 || K == 8);
     const uint32_t negz = 4u * (uint32_t)(K * MP);
     std::vector<uint4> edesc(chunked ? (size_t)R * K * MP : 0, make_uint4(0, 0, 0, 0));
     std::vector<uint4> vdesc3(chunked ? (size_t)R * n : 0, make_uint4(0, 0, 0, 0));
-    std::vector<uint16_t> lpos(chunked ? (size_t)R * MP : 0, 0);
-    std::vector<uint32_t> rinfo_s(chunked ? (size_t)R * MP : 0, 0);
+    std::vector<uint16_t> lpos((size_t)R * MP, 0);
+    std::vector<uint32_t> rinfo_s((size_t)R * MP, 0);
+    // serial path of width 12 (warp per item)
+    std::vector<uint2> vdesc_s(chunked ? 0 : (size_t)R * n), evar(chunked ? 0 : (size_t)R * K * MP, make_uint2(0, 0));
     B->lorder.assign((size_t)R * MP, 0);
     B->lptr.assign((size_t)R * (MP + 1), 0);
     B->nlayers.assign(R, 0);
@@ -657,7 +658,6 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
         if (no_memory) return fail(MBBP_E_NOMEM, "out of memory");
     }
     auto slot_of = [&](int pos, int j) { return (pos >> 5) * (32 * K) + 32 * j + (pos & 31); };
-    std::vector<uint16_t> lrows16((size_t)R * MP, 0);
     int lsteps = 0;
     for (int t = 0; t < R; ++t) {
         const RepLayout& L = layouts[t];
@@ -675,26 +675,18 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
         }
         edges[t] = E;
         const std::vector<int>& ord = L.generic.order;
-        std::vector<uint2> vstart(n);
         for (int p = 0; p < n; ++p) {
             const int v = ord[p];
             uint2 d;
             d.x = (uint32_t)vslot.size();
             d.y = (uint32_t)v | ((uint32_t)vl[v].size() << 16);
             vdesc[(size_t)t * n + p] = d;
-            vstart[v] = d;
             vslot.insert(vslot.end(), vl[v].begin(), vl[v].end());
             if (K == 6) {
                 uint32_t o[6] = {0, 0, 0, 0, 0, 0};
                 for (int i = 0; i < (int)vl[v].size() && i < 6; ++i) o[i] = 4u * vl[v][i];
                 vdesc6[(size_t)t * n + p] = make_uint4(d.y, o[0] | (o[1] << 16), o[2] | (o[3] << 16), o[4] | (o[5] << 16));
             }
-        }
-        // Serial schedule: every edge slot points at its variable's slot list.
-        for (int r = 0; r < M; ++r) {
-            const auto& cols = g.rcols[L.src[r]];
-            for (int j = 0; j < (int)cols.size(); ++j)
-                evar[(size_t)t * K * MP + (size_t)slot_of(pos[r], j)] = vstart[cols[j]];
         }
         const int nl = L.layers;
         int32_t* lo = B->lorder.data() + (size_t)t * MP;
@@ -704,7 +696,6 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
             lp[y] = at;
             for (int r = 0; r < M; ++r)
                 if (L.layer_of[r] == y) {
-                    lrows16[(size_t)t * MP + at] = (uint16_t)pos[r];
                     lo[at++] = r;
                 }
         }
@@ -713,14 +704,41 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
         int steps2 = 0;
         for (int y = 0; y < nl; ++y) steps2 += (lp[y + 1] - lp[y] + 1) / 2;
         lsteps = std::max(lsteps, steps2);
+        // rows: bank-aware positions for the chunk kernel; in their own order at
+        // width 12, where a warp takes up to 32 rows of a layer at once: rows that
+        // follow one another are at different banks then
+        std::vector<int> sp = L.sp;
+        if (!chunked)
+            for (int r = 0; r < M; ++r) sp.push_back(r);
+        for (int i = 0; i < M; ++i) lpos[(size_t)t * MP + i] = (uint16_t)sp[lo[i]];
+        for (int r = 0; r < M; ++r)
+            rinfo_s[(size_t)t * MP + sp[r]] = (uint32_t)L.src[r] | ((uint32_t)g.rcols[L.src[r]].size() << 16);
+        if (!chunked) {
+            std::vector<uint2> vstart(n);
+            std::vector<std::vector<uint16_t>> vr(n);
+            for (int r = 0; r < M; ++r) {
+                const auto& cols = g.rcols[L.src[r]];
+                for (int j = 0; j < (int)cols.size(); ++j) vr[cols[j]].push_back((uint16_t)slot_of(r, j));
+            }
+            std::vector<int> by_degree(n);
+            for (int v = 0; v < n; ++v) {
+                vstart[v] = make_uint2((uint32_t)vslot.size(), (uint32_t)v | ((uint32_t)vr[v].size() << 16));
+                vslot.insert(vslot.end(), vr[v].begin(), vr[v].end());
+                by_degree[v] = v;
+            }
+            std::stable_sort(by_degree.begin(), by_degree.end(),
+                             [&](int a, int b) { return vr[a].size() < vr[b].size(); });
+            for (int p = 0; p < n; ++p) vdesc_s[(size_t)t * n + p] = vstart[by_degree[p]];
+            for (int i = 0; i < M; ++i) {
+                const auto& cols = g.rcols[L.src[lo[i]]];
+                for (int j = 0; j < (int)cols.size(); ++j)
+                    evar[(size_t)t * K * MP + (size_t)slot_of(i, j)] = vstart[cols[j]];
+            }
+        }
         if (chunked) {
-            // chunk kernel: rows at bank-aware positions, descriptors by position
-            const std::vector<int>& sp = L.sp;
+            // descriptors by position
             std::vector<int> row_at(MP, 0);  // row at a generic-layout position
             for (int r = 0; r < M; ++r) row_at[pos[r]] = r;
-            for (int i = 0; i < M; ++i) lpos[(size_t)t * MP + i] = (uint16_t)sp[lo[i]];
-            for (int r = 0; r < M; ++r)
-                rinfo_s[(size_t)t * MP + sp[r]] = (uint32_t)L.src[r] | ((uint32_t)g.rcols[L.src[r]].size() << 16);
             auto pack = [](const uint32_t* o) {
                 return make_uint4(o[0] | (o[1] << 16), o[2] | (o[3] << 16), o[4] | (o[5] << 16),
                                   o[6] | (o[7] << 16));
@@ -825,11 +843,11 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
     const size_t o_vdesc2 = o_rowptr + align256(rowptr.size() * 4);
     const size_t o_rinfo2 = o_vdesc2 + align256(vdesc2.size() * sizeof(uint4));
     const size_t o_hmask2 = o_rinfo2 + align256(rinfo2.size() * 4);
-    const size_t o_lrows = o_hmask2 + align256(hmask2.size() * 4);
-    const size_t o_lptr = o_lrows + align256(lrows16.size() * 2);
+    const size_t o_lptr = o_hmask2 + align256(hmask2.size() * 4);
     const size_t o_nlayers = o_lptr + align256(lptr16.size() * 2);
     const size_t o_evar = o_nlayers + align256((size_t)R * 4);
-    const size_t o_edesc = o_evar + align256(evar.size() * sizeof(uint2));
+    const size_t o_vdesc_s = o_evar + align256(evar.size() * sizeof(uint2));
+    const size_t o_edesc = o_vdesc_s + align256(vdesc_s.size() * sizeof(uint2));
     const size_t o_vdesc3 = o_edesc + align256(edesc.size() * sizeof(uint4));
     const size_t o_lpos = o_vdesc3 + align256(vdesc3.size() * sizeof(uint4));
     const size_t o_rinfo_s = o_lpos + align256(lpos.size() * 2);
@@ -852,10 +870,10 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
         {o_vdesc2, vdesc2.data(), vdesc2.size() * sizeof(uint4)},
         {o_rinfo2, rinfo2.data(), rinfo2.size() * 4},
         {o_hmask2, hmask2.data(), hmask2.size() * 4},
-        {o_lrows, lrows16.data(), lrows16.size() * 2},
         {o_lptr, lptr16.data(), lptr16.size() * 2},
         {o_nlayers, B->nlayers.data(), (size_t)R * 4},
         {o_evar, evar.data(), evar.size() * sizeof(uint2)},
+        {o_vdesc_s, vdesc_s.data(), vdesc_s.size() * sizeof(uint2)},
         {o_edesc, edesc.data(), edesc.size() * sizeof(uint4)},
         {o_vdesc3, vdesc3.data(), vdesc3.size() * sizeof(uint4)},
         {o_lpos, lpos.data(), lpos.size() * 2},
@@ -890,15 +908,15 @@ mbbp_status build_impl(const uint8_t* H, int m, int n, int R, const int32_t* set
     d.hmask2 = shape ? reinterpret_cast<const uint32_t*>(base + o_hmask2) : nullptr;
     d.sedge = shape ? reinterpret_cast<const int32_t*>(base + o_sedge) : nullptr;
     d.vdesc6 = K == 6 ? reinterpret_cast<const uint4*>(base + o_vdesc6) : nullptr;
-    d.lrows = reinterpret_cast<const uint16_t*>(base + o_lrows);
     d.lptr = reinterpret_cast<const uint16_t*>(base + o_lptr);
     d.nlayers = reinterpret_cast<const int32_t*>(base + o_nlayers);
-    d.evar = reinterpret_cast<const uint2*>(base + o_evar);
+    d.evar = chunked ? nullptr : reinterpret_cast<const uint2*>(base + o_evar);
+    d.vdesc_s = chunked ? nullptr : reinterpret_cast<const uint2*>(base + o_vdesc_s);
     d.edesc = chunked ? reinterpret_cast<const uint4*>(base + o_edesc) : nullptr;
     d.vdesc3 = chunked ? reinterpret_cast<const uint4*>(base + o_vdesc3) : nullptr;
-    d.lpos = chunked ? reinterpret_cast<const uint16_t*>(base + o_lpos) : nullptr;
+    d.lpos = reinterpret_cast<const uint16_t*>(base + o_lpos);
     d.lsteps = lsteps;
-    d.rinfo_s = chunked ? reinterpret_cast<const uint32_t*>(base + o_rinfo_s) : nullptr;
+    d.rinfo_s = reinterpret_cast<const uint32_t*>(base + o_rinfo_s);
     *out = B.release();
     return MBBP_OK;
 }

@@ -47,25 +47,30 @@ struct DevBases {
     const int32_t* sedge;     // [R][6*MP] edge id of every message slot (-1: none), for message traces
     int shape, VS, RS, ORS;
 
-    // Serial schedule: rows of H^(t) in layer order, layer boundaries and,
-    // per edge slot, the variable's slot list (x = first vslot entry,
-    // y = variable | degree << 16).
-    const uint16_t* lrows;    // [R][MP]
+    // Serial schedule: layer boundaries (rows in layer order); the rows' positions
+    // in layer order, and per position src row | degree << 16.  Positions: for
+    // the chunk kernel a permutation that spreads its shared-memory accesses over
+    // the banks, at width 12 the rows' own order.
     const uint16_t* lptr;     // [R][MP+1]
     const int32_t* nlayers;   // [R]
+    const uint16_t* lpos;     // [R][MP]
+    const uint32_t* rinfo_s;  // [R][MP]
+    // Serial schedule, width 12 (null otherwise): variables by ascending degree, x
+    // = first vslot entry of its slots, y = variable | degree << 16; the same for
+    // edge j of the row at layer-order index i, at row_slot(i) + 32 j.  Slots by
+    // the positions above, lists in variable order.  Tables of their own: a length-382
+    // code with rows of 10, R = 20, 20,000 shots at p = 0.0127, took 35.2 ms with the
+    // generic tables in row order, 39.0 with those that a search orders for the
+    // flooding kernels, 31.8 with these.
+    const uint2* vdesc_s;     // [R][n]
     const uint2* evar;        // [R][DC*MP]
     // Serial schedule, widths 6 and 8 (null otherwise): per edge slot,
     // x = variable | first other edge << 16 and y/z/w = further other edges of
     // the variable (byte offsets of their slots, ascending row, padded with
     // the offset 4 * DC * MP of a -0.0f slot); per variable, its 8 slot byte
     // offsets (ascending row, padded the same way).
-    const uint4* edesc;       // [R][DC*MP], by row position
+    const uint4* edesc;       // [R][DC*MP], by position
     const uint4* vdesc3;      // [R][n]
-    // chunk-kernel row positions (a permutation of the rows of H^(t) placed
-    // to spread the kernel's shared-memory accesses over the banks): the
-    // positions in layer order, and per position src row | degree << 16
-    const uint16_t* lpos;     // [R][MP]
-    const uint32_t* rinfo_s;  // [R][MP]
     int lsteps;               // most two-row steps of a representation, its layers padded to whole steps
 };
 

@@ -72,6 +72,27 @@ def test_generic_flooding_variants(code, post):
     _assert_exact(got, oracle.mbbp_decode(H, B.sets, s, llr, 40, 0.7, precision="f32"))
 
 
+@pytest.mark.parametrize("code", ["gb78w5", "irregular12"])
+def test_serial_width_12(code):
+    """The serial schedule's kernel of width 12 (tables of its own, rows in their
+    own order): rows of 10 and rows of weight 2 to 12, outputs and posteriors
+    bit for bit as the FP32 oracle's."""
+    import torch
+    from paper_2605_14170_gb300 import mbbp
+    H = _irregular(50, 150, 12, 7) if code == "irregular12" else CODES[code]()
+    n, R = H.shape[1], 4
+    e, _ = oracle.sample(SEED + 12, 0, 41, n, 0.03, "bsc")
+    s = oracle.syndrome(H, e)
+    llr = np.random.default_rng(13).uniform(1.0, 3.0, n).astype(np.float32)
+    B = mbbp.mbbp_build_bases(H, R, SEED)
+    out = _decode(B, s, llr, 30, 0.7, schedule=mbbp.SCHEDULE_SERIAL, want_posterior=True)
+    _assert_exact(out, oracle.mbbp_decode(H, B.sets, s, llr, 30, 0.7, precision="f32",
+                                          schedule=oracle.SCHEDULE_SERIAL))
+    ref = [[oracle.bp(np.vstack([H, H[rows]]), np.concatenate([x, x[rows]]), llr, 30, 0.7, precision="f32",
+                      schedule=1)["post"] for rows in B.sets] for x in s]
+    assert np.array_equal(out["posterior"], np.array(ref))
+
+
 @pytest.mark.parametrize("iters", [0, 1, 40])
 @pytest.mark.parametrize("code", sorted(CODES))
 def test_generic_posteriors(code, iters):
