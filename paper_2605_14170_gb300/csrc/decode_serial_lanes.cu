@@ -138,29 +138,34 @@ __device__ __forceinline__ void lane_posts(int& st, int nw, const int* cend, con
 // call that stays with the warp-per-slot kernel pays 3 to 8 us for both launches:
 // [[72]] R = 4, 20,000 shots at p = 0.001 87 us, 82 without them.
 //
-// Min-sum: rounds * density^2 >= 1 and density >= 0.1, a round being 32 items
-// per SM.  Times as fast as the warp-per-slot kernel (nine or ten codes with rows
-// of weight 6, length 60 to 288, R = 4 to 20, alpha 0.875, 100 iterations;
-// slowest to fastest code), by error rate, density and rounds:
-//      p    density      4         16         32         96
-//   0.001   0.006   0.56-1.99  0.53-1.85      -      0.48-0.97
-//   0.01    0.056   0.73-1.12  0.77-1.12      -      0.88-1.16
-//   0.02    0.11    0.61-1.02  0.71-1.12  0.84-1.29  1.04-1.85
-//   0.04    0.20    0.65-1.14  0.90-1.82  1.03-2.08  1.17-2.52
-//   0.06    0.27    0.77-1.33  1.03-2.19  1.21-2.56  1.47-2.90
-//   0.08    0.32    0.88-1.52  1.22-2.59  1.28-2.85      -
-// Rows of weight 8, irregular rows, alpha 0.625 and limits of 1 to 50 iterations
-// lie higher at the same density.  1.03 is the least of all measured points that
-// satisfy the rule.  Sum-product takes longer in one lane: rounds * density^2 >=
-// 6 and density >= 0.2 (0.20, 64 rounds: 0.97-2.04; 0.32, 16: 0.91-2.00, 64:
-// 1.10-2.44).
+// A call takes this kernel when it has at least 16 rounds (32 items per SM each)
+// and  rounds * density^2 * min(1, density / 0.12) >= c:  the first factors weigh
+// the last shots, whose pace costs up to the iteration limit, so c grows with it,
+// 0.2 + 0.008 iters (min-sum) or 0.5 + 0.1 iters (sum-product, which takes longer
+// in one lane); the last factor weighs the refills, and below densities of 0.05
+// and 0.1 they outweigh all.  Measured at 4,300 points (15 codes of length 60 to
+// 288, rows of weight 2 to 8, R = 1 to 20, error rates 0.003 to 0.2, 1 to 200
+// iterations, 4 to 768 rounds): at the 2,000 that satisfy the rule this kernel is
+// 0.993 to 3.4 times as fast as the warp-per-slot kernel (geometric mean 1.6
+// min-sum, 1.5 sum-product).  Slowest and fastest code, min-sum, 100 iterations,
+// by error rate, density (rows of weight 6) and rounds; [ ] below the rule:
+//      p    density       16             32           96          768
+//   0.003   0.018         -              -       [0.69-0.96]  [0.69-0.98]
+//   0.01    0.057         -              -       [0.88-1.19]   1.03-1.38
+//   0.02    0.11    [0.71-1.12]    [0.84-1.29]    1.04-1.85       -
+//   0.04    0.20    [0.90-1.82]     1.03-2.08     1.17-2.52       -
+//   0.06    0.27     1.03-2.19      1.21-2.56     1.47-2.90       -
+//   0.08    0.32     1.22-2.59      1.28-2.85        -            -
 constexpr int kRouteShots = 128;
 constexpr int kRouteThreads = 1024;
 constexpr int kMinRounds = 16;
 
-float min_density(int rule, double rounds) {
-    return rule == MBBP_RULE_NMS ? std::max(0.1f, (float)std::sqrt(1.0 / rounds))
-                                 : std::max(0.2f, (float)std::sqrt(6.0 / rounds));
+// The least density at which a call takes this kernel.
+float min_density(int rule, int iters, double rounds) {
+    const bool nms = rule == MBBP_RULE_NMS;
+    const double x = (nms ? 0.2 + 0.008 * iters : 0.5 + 0.1 * iters) / rounds;
+    const double d = x >= 0.12 * 0.12 ? std::sqrt(x) : std::cbrt(0.12 * x);
+    return (float)std::max(nms ? 0.05 : 0.1, d);
 }
 
 __global__ void __launch_bounds__(kRouteThreads) serial_route_kernel(const uint8_t* __restrict__ synd, int m, int batch,
@@ -577,7 +582,7 @@ cudaError_t launch_decode_serial_lanes(const DecodeArgs& args, cudaStream_t s, i
     DecodeArgs a = args;
     unsigned int* word = reinterpret_cast<unsigned int*>(a.counter);  // a work counter that this path does not use
     a.lanes = word;
-    serial_route_kernel<<<1, kRouteThreads, 0, s>>>(a.io.synd, B.m, a.io.batch, B.R, min_density(a.rule, rounds), word,
+    serial_route_kernel<<<1, kRouteThreads, 0, s>>>(a.io.synd, B.m, a.io.batch, B.R, min_density(a.rule, a.io.iters, rounds), word,
                                                     a.rep_counter);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
