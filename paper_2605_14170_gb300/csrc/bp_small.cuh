@@ -195,7 +195,7 @@ __device__ __forceinline__ void run_chunk(const DevBases& B, const ShotIO& io, i
         degs |= (dk << (3 * k)) | (__reduce_max_sync(kFull, dk) << (16 + 3 * k));
     }
     // halting-test masks: the first row group's, read every iteration, in
-    // registers (in shared memory, whose path is 92% busy, [[144]] R = 16,
+    // registers (in shared memory, whose path is 89% busy, [[144]] R = 16,
     // 200,000 shots at p = 0.0533 took 21.14 instead of 20.76 ms)
     uint32_t hm0[VS];
 #pragma unroll

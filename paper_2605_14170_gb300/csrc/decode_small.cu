@@ -27,9 +27,11 @@ constexpr int kSmallWarps = 1;  // warps per block: each warp works alone
 // ONCE: every item has a warp of its own (short calls, a decoder in a control
 // loop), which takes the item of its index: no pull, and no counter to clear
 // before the launch.  A kernel of its own: with a test in the loop the one for
-// long calls spills 60 bytes.  [[72,12,6]] R = 4, one shot, ten runs of each
-// (they scatter by up to 18%, the host's part of the call): median 18.3 -> 17.3 us,
-// every one of five pairs faster (by 2.6 to 21%).
+// long calls spills 60 bytes.  [[72,12,6]] R = 4, one shot, both in one process,
+// 30 pairs taken in turn, each faster: median 17.5 -> 16.3 us a call in a row of
+// calls (10% to 90%: 17.2-17.8, 16.1-16.6), 30.5 -> 28.2 us alone, 10.1 -> 4.4 us
+// replayed from a graph; 16 shots 30.9 -> 28.7, 50.4 -> 48.4, 29.2 -> 24.1 us.
+// (Between processes the host's part scatters by up to 18%.)
 struct SmallWork {
     int s8, s2, s1;
 };
